@@ -623,6 +623,17 @@ static lbfe_status copy_columns(lbfe_handle *h, int k, int x0, int nx, char *dev
     const InstDev &I = h->inst[k];
     if (x0 + nx > I.Lx) return LBFE_ERR_BAD_PARAM;
     if (!h->ready[k]) return LBFE_ERR_STATE;
+    // a buffer in this device's memory is copied by one kernel; any other the
+    // copy engine can reach (another device's, pinned host memory) array by array
+    cudaPointerAttributes at;
+    int device = -1;
+    CK(cudaGetDevice(&device));
+    if (cudaPointerGetAttributes(&at, dev) != cudaSuccess)
+        cudaGetLastError();
+    else if (at.type == cudaMemoryTypeDevice && at.device == device) {
+        CK(lbfe::launch_columns(h->ctx(), k, h->cur, x0, nx, dev, get));
+        return LBFE_OK;
+    }
     const size_t rows = (size_t)I.Ly * I.Lz, S = (size_t)I.S;
     const size_t eb = elem_bytes(h->precision);
     auto copy = [&](char *field, size_t esz, size_t count, size_t fstride, size_t &off) -> cudaError_t {

@@ -5,7 +5,8 @@
 //            term) and the Guo velocity u = (j + F/2)/rho (the velocity
 //            field the caller asks for);
 //   init     f = f^eq(rho_s, 0), C = I;
-//   decode / encode of one population array for host copies.
+//   decode / encode of one population array for host copies;
+//   column blocks of the x-split decomposition (all arrays in one launch).
 // The time step itself is the fused kernel (lbfe_fused.cu).  Every instance
 // of a batch is covered by one launch through the tile table (tile_off).
 #include "lbfe_internal.cuh"
@@ -194,7 +195,122 @@ __global__ void k_encode_pop(InstDev I, int cur, int s, int i, const float *src)
     Store<T>::st(f + (long long)(s * Q + i) * I.S + n, v);
 }
 
+// ---------------------------------------------------------------- column blocks
+// Columns [x0, x0 + nx) of every stored array of an instance to or from a
+// contiguous block: populations [38][rows][nx], conformation [6][rows][nx],
+// offset densities [rows][nx] (rows = Ly Lz).  blockIdx.y is the array; the
+// threads of blockIdx.x walk its units of 2^lw bytes, the widest that
+// divides the row and every start (whole rows of a whole lattice are one
+// run of N elements).
+//
+// Bound by HBM for a whole lattice (read and write once) and by its single
+// launch for ghost columns, whose 8-byte rows cost a 32-byte sector each.
+// One 2-D copy per array, the alternative, is 44 (45) launches per block.
+// Measured, 2-D copies -> this kernel: a whole 192 x 96 x 80 FP32 block
+// 0.51 -> 0.12 ms, sixteen of 320 x 44 x 40 4.4 -> 0.5 ms (6.3 TB/s), four
+// steps of two 100-column slabs with their exchanges 10.9 -> 1.35 ms.
+struct ColumnArgs {
+    char *field[3], *block[3];       // populations, conformation, offset densities: first column; block section
+    unsigned long long fstride[3];   // bytes between arrays in the instance
+    unsigned long long bstride[3];   // bytes between arrays in the block
+    int first[4];                    // first array (blockIdx.y) of each section, total
+    int lw[3];                       // log2 bytes of a unit
+    unsigned units[3];               // units of one row of the block
+    unsigned long long pitch[3];     // bytes between rows in the instance
+    unsigned rows;                   // rows of an array (1: one run)
+    int get;
+};
+
+template <typename V>
+__device__ __forceinline__ void copy_units(const ColumnArgs &A, int s, int a) {
+    char *f = A.field[s] + A.fstride[s] * a, *b = A.block[s] + A.bstride[s] * a;
+    const unsigned units = A.units[s];
+    const unsigned long long pitch = A.pitch[s];
+    const unsigned long long total = (unsigned long long)units * A.rows;
+    constexpr int kIlp = 4;          // loads in flight per thread
+    const unsigned long long stride = (unsigned long long)gridDim.x * blockDim.x;
+    for (unsigned long long e0 = (unsigned long long)blockIdx.x * blockDim.x + threadIdx.x; e0 < total;
+         e0 += kIlp * stride) {
+        V v[kIlp];
+        V *dst[kIlp];
+#pragma unroll
+        for (int j = 0; j < kIlp; ++j) {
+            const unsigned long long e = e0 + j * stride;
+            dst[j] = nullptr;
+            if (e >= total) continue;
+            V *pf;
+            if (A.rows == 1) {
+                pf = (V *)f + e;
+            } else {                 // at most 2^26 elements of 8 one-byte units: 32-bit indices
+                const unsigned row = (unsigned)e / units, col = (unsigned)e - row * units;
+                pf = (V *)(f + row * pitch) + col;
+            }
+            V *pb = (V *)b + e;
+            v[j] = A.get ? __ldcs(pf) : __ldcs(pb);
+            dst[j] = A.get ? pb : pf;
+        }
+#pragma unroll
+        for (int j = 0; j < kIlp; ++j)
+            if (dst[j]) *dst[j] = v[j];
+    }
+}
+
+__global__ void __launch_bounds__(kBlock) k_columns(const __grid_constant__ ColumnArgs A) {
+    const int y = blockIdx.y;
+    const int s = y < A.first[1] ? 0 : (y < A.first[2] ? 1 : 2);
+    const int a = y - A.first[s];
+    switch (A.lw[s]) {
+        case 4: copy_units<uint4>(A, s, a); break;
+        case 3: copy_units<uint2>(A, s, a); break;
+        case 2: copy_units<unsigned>(A, s, a); break;
+        case 1: copy_units<unsigned short>(A, s, a); break;
+        default: copy_units<unsigned char>(A, s, a);
+    }
+}
+
 // ---------------------------------------------------------------- launchers
+cudaError_t launch_columns(const LaunchCtx &c, int k, int cur, int x0, int nx, void *block, bool get) {
+    const InstDev &I = c.inst_host[k];
+    const size_t eb = c.precision == LBFE_FP32 ? 4 : 2;
+    const size_t cells = (size_t)nx * I.Ly * I.Lz;
+    const bool whole = nx == I.Lx;
+    ColumnArgs A{};
+    // the current state: f[cur], C[cur] and the offsets f[cur] is stored against
+    char *const field[3] = {(char *)I.f[cur], (char *)I.C[cur], (char *)I.dens[cur ^ 1]};
+    const size_t esz[3] = {eb, sizeof(float), sizeof(float2)};
+    const int count[3] = {2 * Q, 6, c.precision != LBFE_FP32 && I.dens[0] ? 1 : 0};
+    char *b = (char *)block;
+    size_t most = 0;
+    A.rows = whole ? 1u : (unsigned)(I.Ly * I.Lz);
+    A.get = get;
+    for (int s = 0; s < 3; ++s) {
+        A.first[s + 1] = A.first[s] + count[s];
+        if (!count[s]) continue;
+        A.field[s] = field[s] + (size_t)x0 * esz[s];
+        A.block[s] = b;
+        A.fstride[s] = (size_t)I.S * esz[s];
+        A.bstride[s] = cells * esz[s];
+        A.pitch[s] = (size_t)I.Lx * esz[s];
+        const size_t row = (whole ? cells : (size_t)nx) * esz[s];
+        // every start and every step of a unit's address must be a multiple of its width
+        const size_t all = (size_t)A.field[s] | (size_t)A.block[s] | A.fstride[s] | A.bstride[s] | row |
+                           (whole ? 0 : A.pitch[s]);
+        int lw = 4;
+        while (all & (((size_t)1 << lw) - 1)) --lw;
+        A.lw[s] = lw;
+        A.units[s] = (unsigned)(row >> lw);
+        const size_t n = (cells * esz[s]) >> lw;
+        if (n > most) most = n;
+        b += cells * esz[s] * count[s];
+    }
+    // four units per thread, at most about eight waves of blocks over all arrays
+    size_t gx = (most + 4 * kBlock - 1) / (4 * kBlock);
+    const size_t cap = 8 * 8 * 152 / 44;
+    if (gx > cap) gx = cap;
+    k_columns<<<dim3((unsigned)gx, (unsigned)A.first[3]), kBlock, 0, c.stream>>>(A);
+    return cudaGetLastError();
+}
+
 cudaError_t launch_moments(const LaunchCtx &c, int cur) {
     switch (c.precision) {
         case LBFE_FP16_OFFSET: k_moments<__half><<<c.total_tiles, kBlock, 0, c.stream>>>(c.inst_dev, c.tile_off, c.n, cur); break;

@@ -210,6 +210,8 @@ cudaError_t launch_forces(const LaunchCtx &c, int cur);
 cudaError_t launch_init(const LaunchCtx &c, int k, const double *rho_dev, int cur);
 cudaError_t launch_decode_pop(const LaunchCtx &c, int k, int cur, int s, int i, float *dst);
 cudaError_t launch_encode_pop(const LaunchCtx &c, int k, int cur, int s, int i, const float *src);
+// Columns [x0, x0 + nx) of instance k to (get) or from a contiguous device block.
+cudaError_t launch_columns(const LaunchCtx &c, int k, int cur, int x0, int nx, void *block, bool get);
 cudaError_t launch_observables(const LaunchCtx &c, int k, int cur, double *mass_out_dev);
 
 // Host-side droplet analysis (lbfe_analysis.cu): from the observables

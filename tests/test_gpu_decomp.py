@@ -62,3 +62,71 @@ def test_column_blocks_round_trip(L):
     assert np.array_equal(np.delete(f1, range(20, 25), axis=-1), np.delete(f0, range(20, 25), axis=-1))
     with pytest.raises(L.LbfeError):
         s.get_columns(0, p.Lx - 2, 5, t.data_ptr())
+
+
+@pytest.mark.parametrize("prec", [0, 1, 2])
+@pytest.mark.parametrize("x0,nx", [(0, 37), (1, 1), (3, 2), (5, 31), (36, 1)])
+@pytest.mark.parametrize("shift", [0, 2, 1])
+def test_column_blocks_against_the_fields(L, prec, x0, nx, shift):
+    """Blocks of odd lattices, every unit width (whole runs, single columns,
+    buffers at 16-, 2- and 1-byte boundaries): the block holds the stored
+    columns, bit for bit the whole-lattice block's, and comes back intact."""
+    import torch
+    p, _, _ = configs.config1()
+    p = replace(p, Lx=37, Ly=9, Lz=5, precision=prec)
+    rho = 1.0 + np.random.default_rng(nx).uniform(-0.1, 0.1, (2, p.Lz, p.Ly, p.Lx))
+    s = L.Solver(p)
+    s.init(0, rho)
+    s.step(2)
+    eb = 4 if prec == 0 else 2
+
+    def split(raw, n):
+        cells = n * p.Ly * p.Lz
+        f = raw[:38 * cells * eb].reshape(38, p.Lz, p.Ly, n, eb)
+        c = raw[38 * cells * eb:38 * cells * eb + 24 * cells].reshape(6, p.Lz, p.Ly, n, 4)
+        d = raw[38 * cells * eb + 24 * cells:].reshape(-1, p.Lz, p.Ly, n, 8)
+        return f, c, d
+
+    def get(x, n):
+        buf = torch.zeros(s.columns_bytes(0, n) + 16, dtype=torch.uint8, device="cuda")
+        s.get_columns(0, x, n, buf.data_ptr() + shift)
+        torch.cuda.synchronize()
+        assert not buf[:shift].any() and not buf[shift + s.columns_bytes(0, n):].any()
+        return buf, buf.cpu().numpy()[shift:shift + s.columns_bytes(0, n)]
+
+    _, whole = get(0, p.Lx)
+    assert np.array_equal(split(whole, p.Lx)[1].copy().view(np.float32)[..., 0], s.get_field(0, L.FIELD_C))
+    if prec == 0:
+        assert np.array_equal(split(whole, p.Lx)[0].copy().view(np.float32)[..., 0].reshape(2, 19, p.Lz, p.Ly, p.Lx),
+                              s.get_field(0, L.FIELD_F))
+    buf, raw = get(x0, nx)
+    for part, ref in zip(split(raw, nx), split(whole, p.Lx)):
+        assert np.array_equal(part, ref[:, :, :, x0:x0 + nx])
+    # the columns overwritten, then set back: nothing else moves
+    junk = torch.full_like(buf, 60)
+    s.set_columns(0, x0, nx, junk.data_ptr() + shift)
+    for part, ref in zip(split(get(0, p.Lx)[1], p.Lx), split(whole, p.Lx)):
+        keep = np.ones(p.Lx, bool)
+        keep[x0:x0 + nx] = False
+        assert np.array_equal(part[:, :, :, keep], ref[:, :, :, keep])
+        assert (part[:, :, :, x0:x0 + nx] == 60).all()
+    s.set_columns(0, x0, nx, buf.data_ptr() + shift)
+    assert np.array_equal(get(0, p.Lx)[1], whole)
+    s.close()
+
+
+def test_column_blocks_through_pinned_host_memory(L):
+    """A pinned host buffer takes the copy engine's path: same bytes."""
+    import torch
+    p, rho, _ = configs.config1()
+    s = L.Solver(p)
+    s.init(0, rho)
+    s.step(2)
+    n = s.columns_bytes(0, 3)
+    dev = torch.empty(n, dtype=torch.uint8, device="cuda")
+    host = torch.empty(n, dtype=torch.uint8).pin_memory()
+    s.get_columns(0, 4, 3, dev.data_ptr())
+    s.get_columns(0, 4, 3, host.data_ptr())
+    torch.cuda.synchronize()
+    assert torch.equal(dev.cpu(), host)
+    s.close()
