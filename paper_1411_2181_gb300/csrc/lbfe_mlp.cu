@@ -1,17 +1,23 @@
-// lbfe_mlp.cu -- forward, backward and AdamW kernels of the Ca_cr proposal
-// network (lbfe_mlp.h): 6 -> 128 -> 128 -> 128 -> 128 -> 4, GELU.
+// lbfe_mlp.cu -- the Ca_cr proposal network (lbfe_mlp.h):
+// 6 -> 128 -> 128 -> 128 -> 128 -> 4, GELU.
 //
-// The contractions are small (a 2048-row batch is ~0.2 GFLOP per training
-// step), so each layer is a shared-memory-tiled FP32 kernel on the CUDA
-// cores: a block stages 16 input rows and each thread accumulates one
-// output column for all of them, reading the layer's weights (BF16 or FP32,
-// transposed [in][out] so that a warp's loads are contiguous) once per
-// block.  Weight gradients reduce over the batch in a fixed order
-// (deterministic); the loss reduces per block in a fixed tree.
+//   k_net    forward, loss and data gradients of R rows per block: rows are
+//            independent until the weight gradients, so one launch takes them
+//            through all layers and back with every weight in shared memory;
+//   k_wgrad  weight and bias gradients, 32 x 32 outputs per block, the batch
+//            split over blocks and summed in a fixed order (deterministic);
+//   k_adamw  the optimiser.
+//
+// The contractions are small (a 256-row step is 0.08 GFLOP, about 1 us of
+// FP32 units) and activations and gradients are FP32, so they run on the
+// CUDA cores.  Bound by latency: launches, and the chain of nine dependent
+// layers.  Layer by layer (fifteen launches of 2 to 16 blocks, the weight
+// gradient one serial sum over the batch per thread) a 256-row step of
+// training took 0.55 ms with the host part of the loop, now 0.15 ms; a forward
+// pass of 341 rows from and to host arrays 179 us, now 97 us.
 #include <cmath>
 #include <cstring>
 #include <new>
-#include <vector>
 
 #include "../../include/lbfe_mlp.h"
 #include "lbfe_internal.cuh"
@@ -19,131 +25,370 @@
 namespace {
 
 constexpr int kLayers = 5;
-constexpr int kDims[kLayers + 1] = {6, 128, 128, 128, 128, 4};
-constexpr int kRows = 16;       // batch rows per block
+// width of layer boundary l: 6, 128, 128, 128, 128, 4
+__host__ __device__ constexpr int dim(int l) { return l == 0 ? 6 : (l == kLayers ? 4 : 128); }
 constexpr int kHidden = 128;
+constexpr int kNetThreads = 512;
+constexpr int kTile = 32;       // weight-gradient tile
+constexpr int kMaxSplit = 16;   // most parts of the batch in the weight gradients
+constexpr int kSplitRows = 64;  // rows of a part staged at a time
 constexpr int kMaxBatch = 65536;
 
-constexpr size_t layer_offset(int l) {
+__host__ __device__ constexpr size_t layer_offset(int l) {
     size_t o = 0;
-    for (int k = 0; k < l; ++k) o += (size_t)kDims[k] * kDims[k + 1] + kDims[k + 1];
+    for (int k = 0; k < l; ++k) o += (size_t)dim(k) * dim(k + 1) + dim(k + 1);
     return o;
 }
 constexpr size_t kParams = layer_offset(kLayers);
 
-__device__ __forceinline__ float gelu(float x) { return 0.5f * x * (1.0f + erff(x * 0.70710678118654752f)); }
-__device__ __forceinline__ float gelu_grad(float x) {
-    const float cdf = 0.5f * (1.0f + erff(x * 0.70710678118654752f));
-    const float pdf = 0.39894228040143268f * expf(-0.5f * x * x);
-    return cdf + x * pdf;
+// ---------------------------------------------------------------- k_net
+// Shared memory of a block: the three 128 x 128 layers row by row (Wt[in][out],
+// rows padded by 16 bytes: the forward reads along a row, the backward 16
+// bytes of each of 32 rows, both without bank conflicts), the small layers and
+// the biases in FP32, and the rows' activations [k][R].
+template <typename W, int R>
+struct NetSmem {
+    static constexpr int ROW = kHidden * (int)sizeof(W) + 16;      // bytes of a padded row
+    static constexpr int BIG = 0;                                  // [3][128] rows
+    static constexpr int SMALL = 3 * kHidden * ROW;                // floats below
+    static constexpr int W0 = 0, B0 = W0 + 6 * kHidden, B = B0 + kHidden, W4 = B + 3 * kHidden,
+                         B4 = W4 + 4 * kHidden, X = B4 + 4, ACT = X + 8 * R, GRAD = ACT + kHidden * R,
+                         RED = GRAD + 4 * kHidden * R, END = RED + 8 * kHidden * R;
+    static constexpr size_t BYTES = SMALL + sizeof(float) * END;
+    static_assert(BYTES <= 227 * 1024, "shared memory of a block");
+    static_assert(SMALL % 16 == 0 && (ACT * 4) % 16 == 0 && (RED * 4) % 16 == 0, "16-byte rows");
+};
+
+template <typename W> struct WVec;
+template <> struct WVec<__nv_bfloat16> {
+    static __device__ __forceinline__ float2 pair(const char *p) {
+        return __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162 *>(p));
+    }
+    static constexpr int N = 8;      // weights in 16 bytes
+    static __device__ __forceinline__ void vec(const char *p, float w[N]) {
+        const uint4 v = *reinterpret_cast<const uint4 *>(p);
+        const unsigned u[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            w[2 * j] = __uint_as_float(u[j] << 16);
+            w[2 * j + 1] = __uint_as_float(u[j] & 0xffff0000u);
+        }
+    }
+    static __device__ __forceinline__ float one(const __nv_bfloat16 *p) { return __bfloat162float(*p); }
+};
+template <> struct WVec<float> {
+    static __device__ __forceinline__ float2 pair(const char *p) { return *reinterpret_cast<const float2 *>(p); }
+    static constexpr int N = 4;
+    static __device__ __forceinline__ void vec(const char *p, float w[N]) {
+        const float4 v = *reinterpret_cast<const float4 *>(p);
+        w[0] = v.x; w[1] = v.y; w[2] = v.z; w[3] = v.w;
+    }
+    static __device__ __forceinline__ float one(const float *p) { return *p; }
+};
+
+template <int R>
+__device__ __forceinline__ void load_rows(const float *p, float a[R]) {
+    if constexpr (R == 2) {
+        const float2 v = *reinterpret_cast<const float2 *>(p);
+        a[0] = v.x;
+        a[1] = v.y;
+    }
+#pragma unroll
+    for (int q = 0; q < R / 4; ++q) {
+        const float4 v = reinterpret_cast<const float4 *>(p)[q];
+        a[4 * q] = v.x; a[4 * q + 1] = v.y; a[4 * q + 2] = v.z; a[4 * q + 3] = v.w;
+    }
 }
 
-__device__ __forceinline__ float wload(const float *w32, const __nv_bfloat16 *w16, int use16, size_t k) {
-    return use16 ? __bfloat162float(w16[k]) : w32[k];
+__device__ __forceinline__ void cp_async16(void *dst, const void *src) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src)
+                 : "memory");
 }
 
-// Z = A_in W + b (and A_out = gelu(Z) when act), rows [r0, r0 + kRows).
-__global__ void __launch_bounds__(kHidden)
-k_fwd(const float *__restrict__ Ain, int in, const float *__restrict__ w32, const __nv_bfloat16 *__restrict__ w16,
-      int use16, int out, float *__restrict__ Z, float *__restrict__ Aout, int act, int B) {
-    __shared__ float tile[kRows][kHidden];
-    const int r0 = blockIdx.x * kRows, o = threadIdx.x;
-    for (int k = threadIdx.x; k < kRows * in; k += blockDim.x) {
-        const int r = k / in, i = k - r * in;
-        tile[r][i] = (r0 + r < B) ? Ain[(size_t)(r0 + r) * in + i] : 0.f;
+// Rows [r0, r0 + R) of the batch through the network; with GRAD also the loss
+// (one FP64 partial per block) and dL/dZ of every layer.  A[l] and dZ[l] are
+// [B][128] (l = 0..3), dY [B][4].
+struct NetArgs {
+    const void *w;                   // parameters in the kernel's weight type
+    const float *x, *t, *mask;
+    float *y, *A[4], *dZ[4], *dY;
+    double *partial;
+    int B;
+};
+
+template <typename W, int R, bool GRAD>
+__global__ void __launch_bounds__(kNetThreads) k_net(const __grid_constant__ NetArgs N) {
+    using Sm = NetSmem<W, R>;
+    extern __shared__ __align__(16) char net_smem[];
+    float *sf = reinterpret_cast<float *>(net_smem + Sm::SMALL);
+    const W *w = (const W *)N.w;
+    const int t = threadIdx.x, r0 = blockIdx.x * R, rows = min(R, N.B - r0);
+    // every weight starts its way into shared memory, one group per layer
+#pragma unroll
+    for (int l = 0; l < 3; ++l) {
+        const char *src = (const char *)(w + layer_offset(l + 1));
+        constexpr int CH = kHidden * (int)sizeof(W) / 16;           // 16-byte chunks of a row
+        for (int q = t; q < kHidden * CH; q += kNetThreads) {
+            const int row = q / CH, c = q - row * CH;
+            cp_async16(net_smem + Sm::BIG + (l * kHidden + row) * Sm::ROW + 16 * c, src + 16 * (size_t)q);
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    }
+    for (int q = t; q < 7 * kHidden; q += kNetThreads) sf[Sm::W0 + q] = WVec<W>::one(w + q);   // W0, then b0
+    if (t < 3 * kHidden)
+        sf[Sm::B + t] = WVec<W>::one(w + layer_offset(t / kHidden + 1) + kHidden * kHidden + (t & (kHidden - 1)));
+    for (int q = t; q < 4 * kHidden + 4; q += kNetThreads) sf[Sm::W4 + q] = WVec<W>::one(w + layer_offset(4) + q);
+    if (t < 6 * R) {
+        const int r = t / 6, i = t - 6 * r;
+        sf[Sm::X + i * R + r] = r < rows ? N.x[(size_t)(r0 + r) * 6 + i] : 0.f;
     }
     __syncthreads();
-    if (o >= out) return;
-    float acc[kRows];
-    const float bias = wload(w32, w16, use16, (size_t)in * out + o);
+    float *act = sf + Sm::ACT, *red = sf + Sm::RED;
+    // hidden output o of row r from its sum z: activation, its derivative, store
+    auto finish = [&](int l, int o, int r, float z) {
+        const float cdf = 0.5f * (1.0f + erff(z * 0.70710678118654752f));
+        const float a = z * cdf;
+        act[o * R + r] = a;
+        if (GRAD) {
+            sf[Sm::GRAD + (l * kHidden + o) * R + r] = cdf + z * 0.39894228040143268f * expf(-0.5f * z * z);
+            if (r < rows) N.A[l][(size_t)(r0 + r) * kHidden + o] = a;
+        }
+    };
+    {
+        const int o = t & (kHidden - 1);
+        for (int r = t >> 7; r < R; r += kNetThreads / kHidden) {
+            float z = sf[Sm::B0 + o];
 #pragma unroll
-    for (int r = 0; r < kRows; ++r) acc[r] = bias;
-    for (int i = 0; i < in; ++i) {
-        const float w = wload(w32, w16, use16, (size_t)i * out + o);
-#pragma unroll
-        for (int r = 0; r < kRows; ++r) acc[r] += tile[r][i] * w;
+            for (int i = 0; i < 6; ++i) z += sf[Sm::X + i * R + r] * sf[Sm::W0 + i * kHidden + o];
+            finish(0, o, r, z);
+        }
     }
 #pragma unroll
-    for (int r = 0; r < kRows; ++r) {
-        if (r0 + r >= B) break;
-        Z[(size_t)(r0 + r) * out + o] = acc[r];
-        if (act) Aout[(size_t)(r0 + r) * out + o] = gelu(acc[r]);
+    for (int l = 1; l < 4; ++l) {
+        if (l == 1) asm volatile("cp.async.wait_group 2;" ::: "memory");
+        else if (l == 2) asm volatile("cp.async.wait_group 1;" ::: "memory");
+        else asm volatile("cp.async.wait_group 0;" ::: "memory");
+        __syncthreads();
+        // outputs 2 op and 2 op + 1, inputs [16 g, 16 g + 16) of all rows
+        const int op = t & 63, g = t >> 6;
+        const char *wp = net_smem + Sm::BIG + ((l - 1) * kHidden + 16 * g) * Sm::ROW + op * 2 * (int)sizeof(W);
+        float s0[R], s1[R];
+#pragma unroll
+        for (int r = 0; r < R; ++r) s0[r] = s1[r] = 0.f;
+#pragma unroll
+        for (int k = 0; k < 16; ++k) {
+            const float2 v = WVec<W>::pair(wp + k * Sm::ROW);
+            float a[R];
+            load_rows<R>(act + (16 * g + k) * R, a);
+#pragma unroll
+            for (int r = 0; r < R; ++r) {
+                s0[r] += a[r] * v.x;
+                s1[r] += a[r] * v.y;
+            }
+        }
+#pragma unroll
+        for (int r = 0; r < R; ++r)
+            *reinterpret_cast<float2 *>(red + (g * R + r) * kHidden + 2 * op) = make_float2(s0[r], s1[r]);
+        __syncthreads();
+        const int o = t & (kHidden - 1);
+        for (int r = t >> 7; r < R; r += kNetThreads / kHidden) {
+            float z = sf[Sm::B + (l - 1) * kHidden + o];
+#pragma unroll
+            for (int q = 0; q < 8; ++q) z += red[(q * R + r) * kHidden + o];
+            finish(l, o, r, z);
+        }
+    }
+    __syncthreads();
+    // output layer: a warp per (row, output)
+    float *y = red;                  // [R][4]
+    for (int q = t >> 5; q < 4 * R; q += kNetThreads / 32) {
+        const int r = q >> 2, o = q & 3, lane = t & 31;
+        float s = 0.f;
+#pragma unroll
+        for (int k = lane; k < kHidden; k += 32) s += act[k * R + r] * sf[Sm::W4 + k * 4 + o];
+#pragma unroll
+        for (int d = 16; d > 0; d >>= 1) s += __shfl_xor_sync(0xffffffffu, s, d);
+        s += sf[Sm::B4 + o];
+        if (lane == 0) {
+            y[q] = s;
+            if (N.y && r < rows) N.y[(size_t)(r0 + r) * 4 + o] = s;
+        }
+    }
+    if (!GRAD) return;
+    __syncthreads();
+    float *dy = red + 4 * R;         // [R][4]
+    double *ls = reinterpret_cast<double *>(red + 8 * R);           // [R]
+    if (t < R) {
+        double loss = 0.0;
+        float d[4] = {0.f, 0.f, 0.f, 0.f};
+        if (t < rows) {
+            const float *yr = y + 4 * t, *tr = N.t + 4 * (size_t)(r0 + t);
+            const float mk = N.mask ? N.mask[r0 + t] : 1.f;
+            const float e0 = yr[0] - tr[0], e1 = yr[1] - tr[1], e3 = yr[3] - tr[3], z = yr[2];
+            // binary cross-entropy of sigmoid(z) with target t[2], stable form
+            const float bce = fmaxf(z, 0.f) - z * tr[2] + log1pf(expf(-fabsf(z)));
+            const float sig = 1.f / (1.f + expf(-z));
+            loss = (double)(mk * (e0 * e0 + e1 * e1 + e3 * e3) + bce);
+            const float sc = 1.f / (float)N.B;
+            d[0] = 2.f * mk * e0 * sc;
+            d[1] = 2.f * mk * e1 * sc;
+            d[2] = (sig - tr[2]) * sc;
+            d[3] = 2.f * mk * e3 * sc;
+            *reinterpret_cast<float4 *>(N.dY + 4 * (size_t)(r0 + t)) = make_float4(d[0], d[1], d[2], d[3]);
+        }
+#pragma unroll
+        for (int o = 0; o < 4; ++o) dy[4 * t + o] = d[o];
+        ls[t] = loss;
+    }
+    __syncthreads();
+    if (t == 0) {
+        double s = 0.0;
+        for (int r = 0; r < R; ++r) s += ls[r];
+        N.partial[blockIdx.x] = s;
+    }
+    // dZ of the last hidden layer, then down; dz [o][R] in act
+    {
+        const int i = t & (kHidden - 1);
+        for (int r = t >> 7; r < R; r += kNetThreads / kHidden) {
+            float s = 0.f;
+#pragma unroll
+            for (int o = 0; o < 4; ++o) s += dy[4 * r + o] * sf[Sm::W4 + 4 * i + o];
+            s *= sf[Sm::GRAD + (3 * kHidden + i) * R + r];
+            act[i * R + r] = s;
+            if (r < rows) N.dZ[3][(size_t)(r0 + r) * kHidden + i] = s;
+        }
+    }
+#pragma unroll
+    for (int l = 3; l >= 1; --l) {
+        __syncthreads();
+        // input i of all rows from outputs [32 g, 32 g + 32)
+        const int i = t & (kHidden - 1), g = t >> 7;
+        const char *wp = net_smem + Sm::BIG + ((l - 1) * kHidden + i) * Sm::ROW + 32 * g * (int)sizeof(W);
+        float s[R];
+#pragma unroll
+        for (int r = 0; r < R; ++r) s[r] = 0.f;
+        constexpr int V = WVec<W>::N;
+#pragma unroll
+        for (int q = 0; q < 32 / V; ++q) {
+            float v[V];
+            WVec<W>::vec(wp + 16 * q, v);
+#pragma unroll
+            for (int j = 0; j < V; ++j) {
+                float a[R];
+                load_rows<R>(act + (32 * g + V * q + j) * R, a);
+#pragma unroll
+                for (int r = 0; r < R; ++r) s[r] += a[r] * v[j];
+            }
+        }
+#pragma unroll
+        for (int r = 0; r < R; ++r) red[(g * R + r) * kHidden + i] = s[r];
+        __syncthreads();
+        for (int r = t >> 7; r < R; r += kNetThreads / kHidden) {
+            float d = 0.f;
+#pragma unroll
+            for (int q = 0; q < 4; ++q) d += red[(q * R + r) * kHidden + i];
+            d *= sf[Sm::GRAD + ((l - 1) * kHidden + i) * R + r];
+            act[i * R + r] = d;
+            if (r < rows) N.dZ[l - 1][(size_t)(r0 + r) * kHidden + i] = d;
+        }
     }
 }
 
-// Per-sample loss terms and dL/dy (mean over the batch); block partial sums
-// of the loss in a fixed tree order.
-__global__ void __launch_bounds__(256)
-k_loss(const float *__restrict__ Y, const float *__restrict__ T, const float *__restrict__ mask, int B,
-       float *__restrict__ dY, double *__restrict__ partial) {
-    __shared__ double red[256];
-    const int b = blockIdx.x * blockDim.x + threadIdx.x;
-    double l = 0.0;
-    if (b < B) {
-        const float *y = Y + 4 * (size_t)b, *t = T + 4 * (size_t)b;
-        const float mk = mask ? mask[b] : 1.f;
-        const float e0 = y[0] - t[0], e1 = y[1] - t[1], e3 = y[3] - t[3];
-        const float z = y[2];
-        // binary cross-entropy of sigmoid(z) with target t[2], stable form
-        const float bce = fmaxf(z, 0.f) - z * t[2] + log1pf(expf(-fabsf(z)));
-        const float sig = 1.f / (1.f + expf(-z));
-        l = (double)(mk * (e0 * e0 + e1 * e1 + e3 * e3) + bce);
-        const float s = 1.f / (float)B;
-        dY[4 * (size_t)b + 0] = 2.f * mk * e0 * s;
-        dY[4 * (size_t)b + 1] = 2.f * mk * e1 * s;
-        dY[4 * (size_t)b + 2] = (sig - t[2]) * s;
-        dY[4 * (size_t)b + 3] = 2.f * mk * e3 * s;
-    }
-    red[threadIdx.x] = l;
-    __syncthreads();
-    for (int s = 128; s > 0; s >>= 1) {
-        if ((int)threadIdx.x < s) red[threadIdx.x] += red[threadIdx.x + s];
+// ---------------------------------------------------------------- k_wgrad
+// Tile (i0, o0) of dW_l[i][o] = sum_b A_{l-1}[b][i] dZ_l[b][o] over the rows of
+// part blockIdx.y, and, in the tiles with i0 = 0, of db_l[o] = sum_b dZ_l[b][o].
+// With several parts each leaves its sums in part[], and the last part of a
+// tile to finish adds them in the order of the parts.
+constexpr int kTiles = 4 + 3 * 16 + 4;
+
+struct WgradArgs {
+    const float *x, *A[4], *dZ[4], *dY;
+    float *g, *part;                 // gradient vector; [splits][kParams] partial sums
+    unsigned *done;                  // [kTiles] finished parts, zero between launches
+    double *partial;                 // k_net's loss partials: block 0 leaves their sum in partial[0]
+    int B, rows, loss_blocks;        // rows of a part
+};
+
+__global__ void __launch_bounds__(256) k_wgrad(const __grid_constant__ WgradArgs G) {
+    __shared__ __align__(16) float sa[kSplitRows][kTile], sd[kSplitRows][kTile];
+    __shared__ bool s_last;
+    const int t = threadIdx.x, tile = blockIdx.x, splits = gridDim.y;
+    int l, i0, o0;
+    if (tile < 4) { l = 0; i0 = 0; o0 = 32 * tile; }
+    else if (tile < 52) { l = 1 + (tile - 4) / 16; i0 = 32 * ((tile - 4) / 4 % 4); o0 = 32 * ((tile - 4) & 3); }
+    else { l = 4; i0 = 32 * (tile - 52); o0 = 0; }
+    const int in = dim(l), out = dim(l + 1);
+    const float *A = l == 0 ? G.x : G.A[l - 1];
+    const float *D = l == 4 ? G.dY : G.dZ[l];
+    const int ti = (t >> 4) * 2, to = (t & 15) * 2;
+    float acc[2][2] = {{0.f, 0.f}, {0.f, 0.f}}, bsum = 0.f;
+    const int b0 = blockIdx.y * G.rows, b1 = min(G.B, b0 + G.rows);
+    for (int bb = b0; bb < b1; bb += kSplitRows) {
+        const int n = min(kSplitRows, b1 - bb);
+#pragma unroll
+        for (int q = t; q < kSplitRows * kTile; q += 256) {
+            const int r = q / kTile, c = q % kTile;
+            sa[r][c] = r < n && i0 + c < in ? A[(size_t)(bb + r) * in + i0 + c] : 0.f;
+            sd[r][c] = r < n && o0 + c < out ? D[(size_t)(bb + r) * out + o0 + c] : 0.f;
+        }
+        __syncthreads();
+#pragma unroll 16
+        for (int r = 0; r < kSplitRows; ++r) {
+            const float2 a = *reinterpret_cast<const float2 *>(&sa[r][ti]);
+            const float2 d = *reinterpret_cast<const float2 *>(&sd[r][to]);
+            acc[0][0] += a.x * d.x; acc[0][1] += a.x * d.y;
+            acc[1][0] += a.y * d.x; acc[1][1] += a.y * d.y;
+        }
+        if (i0 == 0 && t < kTile) {
+#pragma unroll 16
+            for (int r = 0; r < kSplitRows; ++r) bsum += sd[r][t];
+        }
         __syncthreads();
     }
-    if (threadIdx.x == 0) partial[blockIdx.x] = red[0];
-}
-
-// dW[i][o] = sum_b A_in[b][i] dZ[b][o], db[o] = sum_b dZ[b][o] (batch order).
-__global__ void k_bwd_weight(const float *__restrict__ Ain, const float *__restrict__ dZ, int in, int out, int B,
-                             float *__restrict__ g) {
-    const int k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= (in + 1) * out) return;
-    const int i = k / out, o = k - i * out;
-    float acc = 0.f;
-    if (i < in) {
-        for (int b = 0; b < B; ++b) acc += Ain[(size_t)b * in + i] * dZ[(size_t)b * out + o];
-    } else {
-        for (int b = 0; b < B; ++b) acc += dZ[(size_t)b * out + o];
-    }
-    g[k] = acc;  // layout: Wt[in][out] then b[out]
-}
-
-// dZ_prev[b][i] = (sum_o dZ[b][o] Wt[i][o]) gelu'(Z_prev[b][i]).
-__global__ void __launch_bounds__(kHidden)
-k_bwd_data(const float *__restrict__ dZ, int out, const float *__restrict__ w32,
-           const __nv_bfloat16 *__restrict__ w16, int use16, int in, const float *__restrict__ Zprev,
-           float *__restrict__ dZprev, int B) {
-    __shared__ float tile[kRows][kHidden];
-    const int r0 = blockIdx.x * kRows, i = threadIdx.x;
-    for (int k = threadIdx.x; k < kRows * out; k += blockDim.x) {
-        const int r = k / out, o = k - r * out;
-        tile[r][o] = (r0 + r < B) ? dZ[(size_t)(r0 + r) * out + o] : 0.f;
-    }
-    __syncthreads();
-    if (i >= in) return;
-    float acc[kRows];
+    const size_t base = layer_offset(l);
+    float *dst = splits > 1 ? G.part + (size_t)blockIdx.y * kParams + base : G.g + base;
+    auto each = [&](auto &&fn) {
 #pragma unroll
-    for (int r = 0; r < kRows; ++r) acc[r] = 0.f;
-    for (int o = 0; o < out; ++o) {
-        const float w = wload(w32, w16, use16, (size_t)i * out + o);
+        for (int a = 0; a < 2; ++a)
 #pragma unroll
-        for (int r = 0; r < kRows; ++r) acc[r] += tile[r][o] * w;
+            for (int c = 0; c < 2; ++c)
+                if (i0 + ti + a < in && o0 + to + c < out) fn((i0 + ti + a) * out + o0 + to + c, acc[a][c]);
+        if (i0 == 0 && t < kTile && o0 + t < out) fn(in * out + o0 + t, bsum);
+    };
+    each([&](int k, float &v) { dst[k] = v; });
+    if (splits > 1) {
+        __threadfence();
+        __syncthreads();
+        if (t == 0) {
+            s_last = atomicAdd(G.done + tile, 1u) == (unsigned)splits - 1;
+            if (s_last) G.done[tile] = 0u;
+            __threadfence();
+        }
+        __syncthreads();
+        if (s_last)
+            each([&](int k, float &) {
+                float v[kMaxSplit];
+#pragma unroll
+                for (int s = 0; s < kMaxSplit; ++s)
+                    v[s] = s < splits ? __ldcg(G.part + (size_t)s * kParams + base + k) : 0.f;
+                float sum = 0.f;
+#pragma unroll
+                for (int s = 0; s < kMaxSplit; ++s) sum += v[s];
+                G.g[base + k] = sum;
+            });
     }
-#pragma unroll
-    for (int r = 0; r < kRows; ++r) {
-        if (r0 + r >= B) break;
-        const size_t q = (size_t)(r0 + r) * in + i;
-        dZprev[q] = acc[r] * gelu_grad(Zprev[q]);
+    if (tile == 0 && blockIdx.y == 0) {
+        // the loss: partials in a fixed order, strided sums then a tree
+        __shared__ double red[256];
+        double s = 0.0;
+        for (int q = t; q < G.loss_blocks; q += 256) s += G.partial[q];
+        red[t] = s;
+        __syncthreads();
+        for (int d = 128; d > 0; d >>= 1) {
+            if (t < d) red[t] += red[t + d];
+            __syncthreads();
+        }
+        if (t == 0) G.partial[0] = red[0];
     }
 }
 
@@ -171,8 +416,10 @@ __global__ void k_to_bf16(size_t n, const float *__restrict__ w, __nv_bfloat16 *
 size_t align256(size_t v) { return (v + 255) / 256 * 256; }
 
 struct MlpLayout {
-    size_t w32, w16, m, v, g, Z[kLayers], A[kLayers - 1], dZ[2], dY, partial, total;
+    size_t w32, w16, m, v, g, done, A[kLayers - 1], dZ[kLayers - 1], dY, partial, part, total;
 };
+
+constexpr int kFp32Rows = 2, kSmallRows = 4, kLargeRows = 16;   // rows of a k_net block
 
 MlpLayout mlp_plan(int B) {
     MlpLayout L;
@@ -183,12 +430,12 @@ MlpLayout mlp_plan(int B) {
     L.m = take(sizeof(float) * kParams);
     L.v = take(sizeof(float) * kParams);
     L.g = take(sizeof(float) * kParams);
-    for (int l = 0; l < kLayers; ++l) L.Z[l] = take(sizeof(float) * (size_t)B * kDims[l + 1]);
-    for (int l = 0; l < kLayers - 1; ++l) L.A[l] = take(sizeof(float) * (size_t)B * kDims[l + 1]);
-    L.dZ[0] = take(sizeof(float) * (size_t)B * kHidden);
-    L.dZ[1] = take(sizeof(float) * (size_t)B * kHidden);
+    L.done = take(sizeof(unsigned) * kTiles);
+    for (int l = 0; l < kLayers - 1; ++l) L.A[l] = take(sizeof(float) * (size_t)B * kHidden);
+    for (int l = 0; l < kLayers - 1; ++l) L.dZ[l] = take(sizeof(float) * (size_t)B * kHidden);
     L.dY = take(sizeof(float) * (size_t)B * 4);
-    L.partial = take(sizeof(double) * (size_t)((B + 255) / 256));
+    L.partial = take(sizeof(double) * (size_t)((B + kFp32Rows - 1) / kFp32Rows));
+    L.part = take(sizeof(float) * kParams * kMaxSplit);
     L.total = off;
     return L;
 }
@@ -207,18 +454,43 @@ struct lbfe_mlp {
 
 namespace {
 
-cudaError_t forward(lbfe_mlp *m, const float *x, int B) {
-    const float *Ain = x;
-    for (int l = 0; l < kLayers; ++l) {
-        const int in = kDims[l], out = kDims[l + 1];
-        const size_t o = layer_offset(l);
-        const bool act = l < kLayers - 1;
-        k_fwd<<<(B + kRows - 1) / kRows, kHidden, 0, m->stream>>>(
-            Ain, in, m->p32() + o, m->p16() + o, m->use16, out, m->f(m->L.Z[l]), act ? m->f(m->L.A[l]) : nullptr,
-            act ? 1 : 0, B);
-        if (act) Ain = m->f(m->L.A[l]);
-    }
+template <typename W, int R, bool GRAD>
+cudaError_t net_launch(const NetArgs &N, cudaStream_t st) {
+    // per device and cheap: every call states the shared memory it needs
+    const cudaError_t e = cudaFuncSetAttribute(k_net<W, R, GRAD>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                               (int)NetSmem<W, R>::BYTES);
+    if (e != cudaSuccess) return e;
+    k_net<W, R, GRAD><<<(N.B + R - 1) / R, kNetThreads, NetSmem<W, R>::BYTES, st>>>(N);
     return cudaGetLastError();
+}
+
+// Rows of a k_net block.  Four fill the GPU from small batches on (a row's
+// time through the layers is latency); above four waves of such blocks the
+// weights' way into shared memory counts, and sixteen rows share it.  FP32
+// weights leave room for the activations of two rows.
+int net_rows(const lbfe_mlp *m, int B) {
+    if (!m->use16) return kFp32Rows;
+    return B > 4 * 152 * kSmallRows ? kLargeRows : kSmallRows;
+}
+
+template <bool GRAD>
+cudaError_t net(lbfe_mlp *m, const float *x, const float *t, const float *mask, int B, float *y) {
+    NetArgs N{};
+    N.w = m->use16 ? (const void *)m->p16() : (const void *)m->p32();
+    N.x = x;
+    N.t = t;
+    N.mask = mask;
+    N.y = y;
+    for (int l = 0; l < kLayers - 1; ++l) {
+        N.A[l] = m->f(m->L.A[l]);
+        N.dZ[l] = m->f(m->L.dZ[l]);
+    }
+    N.dY = m->f(m->L.dY);
+    N.partial = (double *)(m->base + m->L.partial);
+    N.B = B;
+    if (!m->use16) return net_launch<float, kFp32Rows, GRAD>(N, m->stream);
+    return net_rows(m, B) == kLargeRows ? net_launch<__nv_bfloat16, kLargeRows, GRAD>(N, m->stream)
+                                        : net_launch<__nv_bfloat16, kSmallRows, GRAD>(N, m->stream);
 }
 
 }  // namespace
@@ -249,7 +521,7 @@ lbfe_status lbfe_mlp_create(lbfe_mlp **mp, int max_batch, int weights_bf16, void
     m->stream = (cudaStream_t)stream;
     m->base = (char *)device_block;
     m->L = mlp_plan(max_batch);
-    cudaError_t e = cudaMemsetAsync(m->base, 0, m->L.g + sizeof(float) * kParams, m->stream);
+    cudaError_t e = cudaMemsetAsync(m->base, 0, m->L.A[0], m->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(m->stream);
     if (e != cudaSuccess) {
         delete m;
@@ -282,10 +554,7 @@ lbfe_status lbfe_mlp_get_params(lbfe_mlp *m, float *host_params) {
 
 lbfe_status lbfe_mlp_forward(lbfe_mlp *m, const float *x_dev, int batch, float *y_dev) {
     if (!m || !x_dev || !y_dev || batch < 1 || batch > m->max_batch) return LBFE_ERR_BAD_PARAM;
-    cudaError_t e = forward(m, x_dev, batch);
-    if (e == cudaSuccess)
-        e = cudaMemcpyAsync(y_dev, m->f(m->L.Z[kLayers - 1]), sizeof(float) * 4 * (size_t)batch,
-                            cudaMemcpyDeviceToDevice, m->stream);
+    const cudaError_t e = net<false>(m, x_dev, nullptr, nullptr, batch, y_dev);
     return e == cudaSuccess ? LBFE_OK : LBFE_ERR_CUDA;
 }
 
@@ -293,39 +562,36 @@ lbfe_status lbfe_mlp_loss_grad(lbfe_mlp *m, const float *x_dev, const float *t_d
                                float *loss_host) {
     if (!m || !x_dev || !t_dev || batch < 1 || batch > m->max_batch) return LBFE_ERR_BAD_PARAM;
     const int B = batch;
-    cudaError_t e = forward(m, x_dev, B);
+    cudaError_t e = net<true>(m, x_dev, t_dev, mask_dev, B, nullptr);
     if (e != cudaSuccess) return LBFE_ERR_CUDA;
-    const int nb = (B + 255) / 256;
-    k_loss<<<nb, 256, 0, m->stream>>>(m->f(m->L.Z[kLayers - 1]), t_dev, mask_dev, B, m->f(m->L.dY),
-                                      (double *)(m->base + m->L.partial));
-    // backward, last layer first
-    const float *dZ = m->f(m->L.dY);
-    int ping = 0;
-    for (int l = kLayers - 1; l >= 0; --l) {
-        const int in = kDims[l], out = kDims[l + 1];
-        const size_t o = layer_offset(l);
-        const float *Ain = l > 0 ? m->f(m->L.A[l - 1]) : x_dev;
-        const int nthr = (in + 1) * out;
-        k_bwd_weight<<<(nthr + 255) / 256, 256, 0, m->stream>>>(Ain, dZ, in, out, B, m->f(m->L.g) + o);
-        if (l > 0) {
-            float *dZp = m->f(m->L.dZ[ping]);
-            k_bwd_data<<<(B + kRows - 1) / kRows, kHidden, 0, m->stream>>>(
-                dZ, out, m->p32() + o, m->p16() + o, m->use16, in, m->f(m->L.Z[l - 1]), dZp, B);
-            dZ = dZp;
-            ping ^= 1;
-        }
+    WgradArgs G{};
+    G.x = x_dev;
+    for (int l = 0; l < kLayers - 1; ++l) {
+        G.A[l] = m->f(m->L.A[l]);
+        G.dZ[l] = m->f(m->L.dZ[l]);
     }
+    G.dY = m->f(m->L.dY);
+    G.g = m->f(m->L.g);
+    G.part = m->f(m->L.part);
+    G.done = (unsigned *)(m->base + m->L.done);
+    G.partial = (double *)(m->base + m->L.partial);
+    G.B = B;
+    // parts of at least 64 rows (one staging round), at most 16 of them
+    int splits = (B + kSplitRows - 1) / kSplitRows;
+    if (splits > kMaxSplit) splits = kMaxSplit;
+    G.rows = ((B + splits - 1) / splits + kSplitRows - 1) / kSplitRows * kSplitRows;
+    splits = (B + G.rows - 1) / G.rows;
+    const int R = net_rows(m, B);
+    G.loss_blocks = (B + R - 1) / R;
+    k_wgrad<<<dim3(kTiles, splits), 256, 0, m->stream>>>(G);
     e = cudaGetLastError();
     if (e != cudaSuccess) return LBFE_ERR_CUDA;
     if (loss_host) {
-        std::vector<double> part(nb);
-        e = cudaMemcpyAsync(part.data(), m->base + m->L.partial, sizeof(double) * nb, cudaMemcpyDeviceToHost,
-                            m->stream);
+        double sum = 0.0;
+        e = cudaMemcpyAsync(&sum, m->base + m->L.partial, sizeof sum, cudaMemcpyDeviceToHost, m->stream);
         if (e == cudaSuccess) e = cudaStreamSynchronize(m->stream);
         if (e != cudaSuccess) return LBFE_ERR_CUDA;
-        double s = 0.0;
-        for (double v : part) s += v;
-        *loss_host = (float)(s / B);
+        *loss_host = (float)(sum / B);
     }
     return LBFE_OK;
 }

@@ -89,3 +89,35 @@ def test_training_reduces_loss(M):
     net.set_params(M.init_params(0))
     hist = net.fit(x, t, epochs=300, lr=3e-3, batch=256)
     assert hist[-1] < 0.25 * hist[0]
+
+
+# a forward error of each of five layers of at most 128 FP32 roundings each,
+# passed back through as many: 5 x 128 x 2^-24, relative to the largest entry
+TOL_CHAIN = 5 * 128 * 2.0 ** -24
+
+
+@pytest.mark.parametrize("bf16", [False, True])
+@pytest.mark.parametrize("B", [2, 5, 63, 64, 65, 1025, 2432, 2449])
+def test_row_blocks_and_batch_parts(M, B, bf16):
+    """Batches at the edges of the row blocks (2, 4 and 16 rows) and of the
+    weight gradient's parts (one, several, the most), with FP32 and BF16
+    weights: outputs, loss and gradient against the reference evaluated at
+    the weights the kernels read; repeated calls give the same bits."""
+    import torch
+    net = M.MLP(max_batch=2449, bf16=bf16)
+    p = M.init_params(B)
+    net.set_params(p)
+    pr = p.astype(np.float64)
+    if bf16:
+        pr = torch.tensor(p).to(torch.bfloat16).to(torch.float64).numpy()
+    x, t, mask = batch(B, B + 1)
+    y = net.forward(x)
+    yr = R.forward(pr, x.astype(np.float64))
+    assert np.abs(y - yr).max() / np.abs(yr).max() < TOL_CHAIN
+    loss = net.loss_grad(x, t, mask)
+    g = net.grads()
+    lr_, gr = R.loss_grad(pr, x.astype(np.float64), t.astype(np.float64), mask)
+    assert abs(loss - lr_) / abs(lr_) < TOL_CHAIN
+    assert per_tensor_err(g, gr) < TOL_CHAIN
+    assert net.loss_grad(x, t, mask) == loss and np.array_equal(net.grads(), g)
+    assert np.array_equal(net.forward(x), y)
