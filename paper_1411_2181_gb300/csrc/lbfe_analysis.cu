@@ -108,6 +108,11 @@ void sym_eig3(const double M[6], double ev[3], double V[3][3]) {
     for (int i = 0; i < 3; ++i) ev[i] = A[i][i];
 }
 
+void masses_from_record(const unsigned long long *record, int Lx, lbfe_obs *out) {
+    std::memcpy(out->mass, record + 6 * (size_t)Lx, sizeof out->mass);
+    out->flags = (int)record[6 * (size_t)Lx + 2];
+}
+
 void droplet_from_profile(const unsigned long long *prof, int Lx, double R, lbfe_obs *out) {
     std::vector<long long> A(Lx);
     for (int x = 0; x < Lx; ++x) A[x] = (long long)prof[x];

@@ -16,10 +16,6 @@
 
 #include "lbfe_internal.cuh"
 
-namespace lbfe {
-cudaError_t obs_set_smem_limit(size_t bytes);
-}
-
 using lbfe::InstDev;
 
 namespace {
@@ -91,7 +87,7 @@ lbfe_status derive(const lbfe_params &p, Derived &d) {
 }
 
 struct Layout {
-    size_t inst_off, tile_off, item_off, status_off, mass_off, maps_off;
+    size_t inst_off, tile_off, item_off, status_off, maps_off;
     std::vector<size_t> f_off[2], C_off[2], scratch_off, prof_off, mpart_off, dens_off;
     size_t total;
 };
@@ -111,7 +107,6 @@ Layout plan(const lbfe_params *p, int n) {
     // launch word, work counters, then one status word per instance and
     // two step-count words per instance (by ping-pong parity)
     L.status_off = take(sizeof(unsigned) * (4 + 3 * (size_t)n));
-    L.mass_off = take(sizeof(double) * 2);
     L.maps_off = take(sizeof(lbfe::StepMaps) * 2 * (size_t)n);   // TMA maps, [instance][parity]
     const size_t eb = elem_bytes(p[0].precision);
     for (int k = 0; k < n; ++k) {
@@ -121,7 +116,7 @@ Layout plan(const lbfe_params *p, int n) {
         L.C_off[0].push_back(take(sizeof(float) * 6 * S));
         L.C_off[1].push_back(take(sizeof(float) * 6 * S));
         L.scratch_off.push_back(take(sizeof(float) * 14 * S));
-        L.prof_off.push_back(take(sizeof(unsigned long long) * 6 * (size_t)p[k].Lx));
+        L.prof_off.push_back(take(sizeof(unsigned long long) * lbfe::obs_words(p[k].Lx)));
         L.mpart_off.push_back(take(sizeof(double) * 2 * lbfe::kObsBlocks));
         // reduced storage forms: per-cell offset densities, ping-pong
         L.dens_off.push_back(p[0].precision == LBFE_FP32 ? 0 : take(sizeof(float) * 2 * 2 * S));
@@ -153,7 +148,6 @@ struct lbfe_handle {
     int advection = 0;               // lbfe_params::advection of every instance
     unsigned inject = 0;             // lbfe_test_inject bits
     unsigned *status = nullptr;
-    double *mass = nullptr;
     int cur = 0;
     // CUDA graphs of one time step from each parity of the ping-pong state,
     // captured on a private stream and replayed by lbfe_step; dropped when
@@ -346,10 +340,8 @@ lbfe_status lbfe_create(lbfe_handle **hp, const lbfe_params *p, int n, void *dev
     h->tile_off = (int *)(h->base + L.tile_off);
     h->item_off = (int *)(h->base + L.item_off);
     h->status = (unsigned *)(h->base + L.status_off);
-    h->mass = (double *)(h->base + L.mass_off);
     h->maps_dev = (lbfe::StepMaps *)(h->base + L.maps_off);
     std::vector<int> toff(n + 1, 0);
-    int maxLx = 0;
     for (int k = 0; k < n; ++k) {
         Derived d;
         derive(p[k], d);
@@ -388,15 +380,12 @@ lbfe_status lbfe_create(lbfe_handle **hp, const lbfe_params *p, int n, void *dev
         }
         h->inst.push_back(I);
         toff[k + 1] = toff[k] + (int)((I.N + lbfe::kBlock - 1) / lbfe::kBlock);
-        if (p[k].Lx > maxLx) maxLx = p[k].Lx;
     }
     h->total_tiles = toff[n];
     cudaError_t e = cudaMemcpyAsync(h->inst_dev, h->inst.data(), sizeof(InstDev) * n, cudaMemcpyHostToDevice, h->stream);
     if (e == cudaSuccess) e = cudaMemcpyAsync(h->tile_off, toff.data(), sizeof(int) * (n + 1), cudaMemcpyHostToDevice, h->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(h->status, 0, sizeof(unsigned) * (4 + 3 * (size_t)n), h->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
-    const size_t smem = sizeof(unsigned long long) * 6 * (size_t)maxLx;
-    if (e == cudaSuccess && smem > 48 * 1024) e = lbfe::obs_set_smem_limit(smem);
     int dev = 0;
     if (e == cudaSuccess) e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&h->num_sms, cudaDevAttrMultiProcessorCount, dev);
@@ -490,24 +479,19 @@ lbfe_status lbfe_observables(lbfe_handle *h, int k, lbfe_obs *out) {
     if (!h->ready[k]) return LBFE_ERR_STATE;
     const InstDev &I = h->inst[k];
     const lbfe_params &p = h->params[k];
-    CK(lbfe::launch_observables(h->ctx(), k, h->cur, h->mass));
-    std::vector<unsigned long long> prof(6 * (size_t)I.Lx);
-    double mass[2];
-    unsigned st = 0;
-    CK(cudaMemcpyAsync(prof.data(), I.prof, sizeof(unsigned long long) * prof.size(), cudaMemcpyDeviceToHost, h->stream));
-    CK(cudaMemcpyAsync(mass, h->mass, sizeof mass, cudaMemcpyDeviceToHost, h->stream));
-    CK(cudaMemcpyAsync(&st, I.status, sizeof st, cudaMemcpyDeviceToHost, h->stream));
+    CK(lbfe::launch_observables(I, h->precision, h->cur, h->status, h->stream));
+    std::vector<unsigned long long> rec(lbfe::obs_words(I.Lx));
+    CK(cudaMemcpyAsync(rec.data(), I.prof, sizeof(unsigned long long) * (rec.size() - 1), cudaMemcpyDeviceToHost,
+                       h->stream));
     CK(cudaStreamSynchronize(h->stream));
 
     memset(out, 0, sizeof *out);
     out->step = h->steps[k];
-    out->mass[0] = mass[0];
-    out->mass[1] = mass[1];
-    out->flags = (int)st;
+    lbfe::masses_from_record(rec.data(), I.Lx, out);
     const double tem = p.sigma > 0 ? p.R * p.eta_M / p.sigma : 0.0;
     out->t_over_tem = tem > 0 ? (double)h->steps[k] / tem : 0.0;
-    lbfe::droplet_from_profile(prof.data(), I.Lx, p.R, out);
-    return (st & lbfe::kFlagDiverged) ? LBFE_ERR_DIVERGED : LBFE_OK;
+    lbfe::droplet_from_profile(rec.data(), I.Lx, p.R, out);
+    return (out->flags & (int)lbfe::kFlagDiverged) ? LBFE_ERR_DIVERGED : LBFE_OK;
 }
 
 lbfe_status lbfe_get_field(lbfe_handle *h, int k, int which, void *host_dst, size_t bytes) {

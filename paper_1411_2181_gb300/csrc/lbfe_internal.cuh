@@ -102,7 +102,7 @@ struct InstDev {
     float *jm;                       // scratch [3][S] total momentum
     float *u;                        // scratch [3][S]
     float *F;                        // scratch [2][3][S] per-component total force
-    unsigned long long *prof;        // observables: [6][Lx] per-plane integer sums
+    unsigned long long *prof;        // observables: record of obs_words(Lx) words (lbfe_obs.cu)
     double *mpart;                   // observables: [2][kObsBlocks] mass partials
     float G, Uw, nu_A, nu_B;         // Shan-Chen coupling, wall speed, solvent viscosities
     float pi_coef, L2, inv_tauP;     // eta_P/tau_P, L^2, 1/tau_P
@@ -123,7 +123,10 @@ __device__ __forceinline__ void raise_flag(unsigned *global, const InstDev &I, u
 
 constexpr int kBlock = 256;          // threads per block of the cell-per-thread kernels
 constexpr int kMaxLx = 4096;         // largest Lx lbfe_derive accepts
-constexpr int kObsBlocks = 304;      // 2 x 152 SMs for the observables reduction
+constexpr int kObsBlocks = 608;      // 4 x 152 SMs for the observables reduction
+static_assert(kObsBlocks >= (kMaxLx + 31) / 32, "a block per 32 x-planes");
+// Observables record: 6 Lx plane sums, the masses, the status word, a counter.
+__host__ __device__ constexpr size_t obs_words(int Lx) { return 6 * (size_t)Lx + 4; }
 
 __device__ __forceinline__ int wrapi(int a, int L) { return a < 0 ? a + L : (a >= L ? a - L : a); }
 
@@ -212,11 +215,12 @@ cudaError_t launch_decode_pop(const LaunchCtx &c, int k, int cur, int s, int i, 
 cudaError_t launch_encode_pop(const LaunchCtx &c, int k, int cur, int s, int i, const float *src);
 // Columns [x0, x0 + nx) of instance k to (get) or from a contiguous device block.
 cudaError_t launch_columns(const LaunchCtx &c, int k, int cur, int x0, int nx, void *block, bool get);
-cudaError_t launch_observables(const LaunchCtx &c, int k, int cur, double *mass_out_dev);
+cudaError_t launch_observables(const InstDev &I, int precision, int cur, unsigned *status, cudaStream_t stream);
 
 // Host-side droplet analysis (lbfe_analysis.cu): from the observables
 // kernel's per-plane sums prof[6][Lx], fill L_p, L_p/2R, necks, fragments,
 // broken, volume, centroid, M, D and theta of out.
+void masses_from_record(const unsigned long long *record, int Lx, lbfe_obs *out);   // masses and flags
 void droplet_from_profile(const unsigned long long *prof, int Lx, double R, lbfe_obs *out);
 void sym_eig3(const double M[6], double ev[3], double V[3][3]);
 

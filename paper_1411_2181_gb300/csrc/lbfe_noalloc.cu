@@ -7,18 +7,14 @@
 // start-up, or they cannot afford the device-wide synchronisation that
 // cudaFree implies in a latency-sensitive loop.  For them this entry point
 // computes the observables of a population field they already hold, with
-// its scratch (the per-plane sums, the mass partials, the status word and a
-// copy of the field descriptor) in a file-scope device array that every GPU
+// its scratch (the observables record, the mass partials and the status
+// word) in a file-scope device array that every GPU
 // loading this library keeps until the process exits.  It calls no
 // cudaMalloc, cudaFree or other allocating routine.
 #include <cstring>
 #include <mutex>
 
 #include "lbfe_internal.cuh"
-
-namespace lbfe {
-cudaError_t obs_set_smem_limit(size_t bytes);
-}
 
 namespace {
 
@@ -29,15 +25,12 @@ static_assert(kScratchMaxLx >= lbfe::kMaxLx, "static scratch smaller than the ac
 constexpr int kMaxDevices = 64;
 
 // Layout of the static scratch (8-byte words):
-//   [0, 6*kScratchMaxLx)           per-plane integer sums
+//   [0, obs_words(kScratchMaxLx))  observables record (per-plane sums, masses, status)
 //   next 2*kObsBlocks              FP64 mass partials
-//   next 2                          FP64 masses
 //   next 1                          status word (low 32 bits)
-//   next ceil(sizeof(InstDev)/8)    field descriptor
-constexpr size_t kProfWords = 6 * (size_t)kScratchMaxLx;
+constexpr size_t kProfWords = lbfe::obs_words(kScratchMaxLx);
 constexpr size_t kPartWords = 2 * (size_t)lbfe::kObsBlocks;
-constexpr size_t kDescWords = (sizeof(lbfe::InstDev) + 7) / 8;
-constexpr size_t kScratchWords = kProfWords + kPartWords + 2 + 1 + kDescWords;
+constexpr size_t kScratchWords = kProfWords + kPartWords + 1;
 
 static __device__ __align__(256) unsigned long long g_noalloc_scratch[kScratchWords];
 
@@ -94,39 +87,18 @@ extern "C" lbfe_status lbfe_observables_noalloc(const lbfe_params *p, const void
     I.mpart = (double *)(words + kProfWords);
     I.rho0[0] = (float)p->rho0[0];
     I.rho0[1] = (float)p->rho0[1];
-    double *mass_dev = (double *)(words + kProfWords + kPartWords);
-    unsigned *status_dev = (unsigned *)(words + kProfWords + kPartWords + 2);
-    lbfe::InstDev *desc_dev = (lbfe::InstDev *)(words + kProfWords + kPartWords + 3);
-
-    lbfe::LaunchCtx c;
-    memset(&c, 0, sizeof c);
-    c.inst_dev = desc_dev;
-    c.inst_host = &I;
-    c.n = 1;
-    c.precision = p->precision;
-    c.status = status_dev;
-    c.stream = s;
+    unsigned *status_dev = (unsigned *)(words + kProfWords + kPartWords);
     cudaError_t e = cudaMemsetAsync(status_dev, 0, sizeof(unsigned long long), s);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(desc_dev, &I, sizeof I, cudaMemcpyHostToDevice, s);
-    if (e == cudaSuccess) {
-        const size_t smem = sizeof(unsigned long long) * 6 * (size_t)p->Lx;
-        if (smem > 48 * 1024) e = lbfe::obs_set_smem_limit(smem);
-    }
-    if (e == cudaSuccess) e = lbfe::launch_observables(c, 0, 0, mass_dev);  // clears the plane sums itself
-    double mass[2] = {0.0, 0.0};
-    unsigned status = 0;
     if (e == cudaSuccess)
-        e = cudaMemcpyAsync(g_host_prof, words, sizeof(unsigned long long) * 6 * (size_t)p->Lx,
+        e = lbfe::launch_observables(I, p->precision, 0, status_dev, s);  // clears the record itself
+    if (e == cudaSuccess)
+        e = cudaMemcpyAsync(g_host_prof, words, sizeof(unsigned long long) * (lbfe::obs_words(p->Lx) - 1),
                             cudaMemcpyDeviceToHost, s);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(mass, mass_dev, sizeof mass, cudaMemcpyDeviceToHost, s);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(&status, status_dev, sizeof status, cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
     if (e != cudaSuccess) return LBFE_ERR_CUDA;
 
     memset(out, 0, sizeof *out);
-    out->mass[0] = mass[0];
-    out->mass[1] = mass[1];
-    out->flags = (int)status;
+    lbfe::masses_from_record(g_host_prof, p->Lx, out);
     lbfe::droplet_from_profile(g_host_prof, p->Lx, p->R, out);
-    return (status & lbfe::kFlagDiverged) ? LBFE_ERR_DIVERGED : LBFE_OK;
+    return (out->flags & (int)lbfe::kFlagDiverged) ? LBFE_ERR_DIVERGED : LBFE_OK;
 }
