@@ -187,10 +187,43 @@ struct lbfe_handle {
     }
 };
 
+// Depth of the z-chunks: the one with the fewest planes marched by the busiest
+// block (a chunk costs four planes more than it holds).  Items of one lattice
+// are equal and start together, so that they march in waves of the resident
+// blocks; the items of a batch are handed out as blocks become free, and what
+// that leaves uneven came to about two items (below: 523, 485 and 438 planes'
+// time at 93, 49 and 27 planes a chunk).  Chunks of at least 8 planes.
+// Measured, us per step, chunks that fill the blocks about once -> this:
+// 256 x 128 x 64 FP16 (12 rows; 88 columns) 307 -> 212, twelve uneven lattices
+// FP16 2234 -> 1870; 192 x 96 x 80 keeps its 40 (FP32) and 27 planes (FP16).
+static int auto_z_chunk(const std::vector<InstDev> &inst, long long slots) {
+    int lz = 0, best = 8;
+    for (auto &I : inst) lz = std::max(lz, I.Lz);
+    double best_cost = 0.0;
+    for (int zc = std::max(8, lz); zc >= 8; --zc) {
+        long long items = 0, planes = 0;
+        int deepest = 0;
+        for (auto &I : inst) {
+            const int c = std::min(zc, I.Lz);
+            const long long col = (long long)I.ntx * I.nty, nz = (I.Lz + c - 1) / c;
+            items += col * nz;
+            planes += col * (I.Lz + 4 * nz);
+            deepest = std::max(deepest, c + 4);
+        }
+        double cost = deepest;
+        if (items > slots)
+            cost = inst.size() == 1 ? (double)deepest * ((items + slots - 1) / slots)
+                                    : (double)planes / slots + 2.0 * deepest;
+        if (best_cost == 0.0 || cost < best_cost) {
+            best_cost = cost;
+            best = zc;
+        }
+    }
+    return best;
+}
+
 // Work items of the fused kernel: per instance ceil(Lx/32) x ceil(Ly/TY)
-// column tiles times nzc z-chunks.  Without a requested chunk depth, nzc is
-// chosen so that the items fill the resident blocks of the GPU about once
-// (chunks of at least 8 planes).
+// column tiles times nzc z-chunks, of the requested depth or auto_z_chunk's.
 static lbfe_status configure_fused(lbfe_handle *h, int step_kernel, int tile_y, int z_chunk) {
     if (step_kernel == LBFE_STEP_PAIR) {
         if (tile_y != 16) return LBFE_ERR_BAD_PARAM;
@@ -206,23 +239,16 @@ static lbfe_status configure_fused(lbfe_handle *h, int step_kernel, int tile_y, 
     cudaError_t e = lbfe::fused_prepare(step_kernel, tile_y, h->precision, h->advection, &bps);
     if (e != cudaSuccess) return cuda_fail(e, "fused_prepare");
     if (bps < 1) return LBFE_ERR_BAD_PARAM;
-    long long columns = 0;
     for (auto &I : h->inst) {
         I.ntx = (I.Lx + 31) / 32;
         I.nty = (I.Ly + tile_y - 1) / tile_y;
-        columns += (long long)I.ntx * I.nty;
     }
     const long long slots = (long long)h->num_sms * bps;
+    const int zc_auto = z_chunk == 0 ? auto_z_chunk(h->inst, slots) : 0;
     std::vector<int> off(h->n + 1, 0);
     for (int k = 0; k < h->n; ++k) {
         InstDev &I = h->inst[k];
-        int zc = z_chunk;
-        if (zc == 0) {
-            long long nz = (slots + columns / 2) / columns;
-            if (nz < 1) nz = 1;
-            zc = (int)((I.Lz + nz - 1) / nz);
-            if (zc < 8) zc = 8;
-        }
+        int zc = z_chunk == 0 ? zc_auto : z_chunk;
         if (zc > I.Lz) zc = I.Lz;
         I.zc = zc;
         I.nzc = (I.Lz + zc - 1) / zc;
