@@ -181,8 +181,9 @@ lbfe_status lbfe_init(lbfe_handle *h, int k, const double *rho_init);
  * moving walls of Sec. 3, coupled to the finite-difference FENE-P update of
  * C (Eqs. 2 and 4) and to the polymer-stress divergence of Eqs. 1 and 3),
  * asynchronously on the stream.
- * With nsteps >= 2 the steps replay CUDA graphs of one step (captured once
- * per launch shape on a private stream); results are identical to single
+ * With nsteps >= 2 the tile kernels' steps replay CUDA graphs of one step
+ * (captured once per launch shape on a private stream), and the three-pass
+ * kernel takes up to 16 steps in a launch; results are identical to single
  * steps.  Inside a stream capture of the caller the kernels are launched
  * directly into it. */
 lbfe_status lbfe_step(lbfe_handle *h, long long nsteps);
@@ -229,11 +230,14 @@ lbfe_status lbfe_set_columns(lbfe_handle *h, int k, int x0, int nx, const void *
  * its parameter space). */
 int lbfe_launches_per_step(const lbfe_handle *h);
 
-/* Variants of the time-step kernel.  Both compute the same step (results
- * agree to FP32 rounding); they differ in speed only. */
+/* Variants of the time-step kernel.  All compute the same step (results
+ * agree to FP32 rounding, CELL and PASSES bit for bit); they differ in speed
+ * only. */
 typedef enum {
     LBFE_STEP_CELL = 0,   /* one cell per thread, tiles of 32 x tile_y cells, tile_y in {8, 12, 16} */
-    LBFE_STEP_PAIR = 1    /* two x-adjacent cells per thread, 32 x 16 tiles; needs even Lx everywhere */
+    LBFE_STEP_PAIR = 1,   /* two x-adjacent cells per thread, 32 x 16 tiles; needs even Lx everywhere */
+    LBFE_STEP_PASSES = 2  /* three passes over the lattice in memory order, several steps per launch;
+                             tile_y 8 and z_chunk 0 */
 } lbfe_step_kernel;
 
 /* Launch shape of the step kernel: variant (lbfe_step_kernel), column-tile
@@ -241,14 +245,16 @@ typedef enum {
  * planes (0 = automatic: fill the resident blocks of the GPU about once).
  * A new handle starts with LBFE_STEP_CELL, tile_y 8 (FP32, or any precision
  * with LBFE_ADVECTION_UPWIND2_MINMOD) or 12 (FP16 / BF16 storage) and the
- * automatic z-chunk.  With LBFE_ADVECTION_UPWIND2_MINMOD only
+ * automatic z-chunk, and takes LBFE_STEP_PASSES by itself where that is
+ * faster for its lattices (small, ragged or many): the fields are the same
+ * bit for bit.  A handle that was tuned keeps what it was given.  With LBFE_ADVECTION_UPWIND2_MINMOD only
  * LBFE_STEP_CELL at tile_y 8 is accepted.
  * LBFE_ERR_BAD_PARAM for an unsupported combination.  Synchronises the
  * stream. */
 lbfe_status lbfe_tune(lbfe_handle *h, int step_kernel, int tile_y, int z_chunk);
-/* Current launch shape (any output may be NULL): kernel variant, tile
- * height, z-chunk of instance 0, persistent grid size and number of work
- * items. */
+/* Current launch shape of the tile kernels (any output may be NULL): kernel
+ * variant, tile height, z-chunk of instance 0, persistent grid size and number
+ * of work items. */
 lbfe_status lbfe_launch_config(const lbfe_handle *h, int *step_kernel, int *tile_y, int *z_chunk, int *grid,
                                int *items);
 
@@ -266,6 +272,12 @@ lbfe_status lbfe_launch_config(const lbfe_handle *h, int *step_kernel, int *tile
  * (Lx * element size a multiple of 16 bytes) wait.  what = 0 restores the
  * maps.  Synchronises the stream; BAD_PARAM for unknown bits. */
 #define LBFE_INJECT_SHORT_COPIES 1u
+/* what = LBFE_INJECT_LOST_COUNTS: with LBFE_STEP_PASSES the first pass of a
+ * step is not counted as finished, so that the second pass's bounded waits for
+ * it expire (about one second); every team then runs through its slots without
+ * waiting and lbfe_check reports LBFE_ERR_TIMEOUT.  SHORT_COPIES makes the
+ * handle step with the tile kernels. */
+#define LBFE_INJECT_LOST_COUNTS 2u
 lbfe_status lbfe_test_inject(lbfe_handle *h, unsigned what);
 
 /* Observables of a population field the caller already holds on the

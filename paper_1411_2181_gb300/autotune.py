@@ -2,9 +2,9 @@
 
 The step kernel runs one block per column tile and z-chunk, in one of two
 variants: one cell per thread with tiles of 32 x TY cells (TY = 8, 12 or 16)
-or two x-adjacent cells per thread with 32 x 16 tiles (even Lx only).  The
-variant, tile height and chunk depth change speed only (the fields agree to
-FP32 rounding).  ``tune`` times each candidate on a scratch solver built
+or two x-adjacent cells per thread with 32 x 16 tiles (even Lx only); or in
+three passes over the lattice in memory order.  The variant, tile height and
+chunk depth change speed only (the fields agree to FP32 rounding).  ``tune`` times each candidate on a scratch solver built
 from the same parameters, keeps the fastest, and caches the choice in a JSON
 file keyed by the GPU name, the precision and the lattice sizes of the
 batch.
@@ -25,7 +25,7 @@ CACHE = os.path.join(os.path.dirname(os.path.abspath(__file__)), "_build", "auto
 
 def _key(params: list[Params], gpu: str) -> str:
     dims = ";".join(f"{p.Lx}x{p.Ly}x{p.Lz}" for p in params)
-    return f"{gpu}|v2|prec{params[0].precision}|adv{params[0].advection}|n{len(params)}|{dims}"
+    return f"{gpu}|v3|prec{params[0].precision}|adv{params[0].advection}|n{len(params)}|{dims}"
 
 
 def _load(path):
@@ -39,7 +39,8 @@ def _load(path):
 def candidates(params: list[Params]):
     """(kernel, tile_y, z_chunk) triples: cell kernel (0) at every tile
     height, pair kernel (1) at 16 rows when every Lx is even; with the
-    second-order advection scheme the cell kernel at 8 rows only."""
+    second-order advection scheme the cell kernel at 8 rows only.  The
+    three-pass kernel (2) has one shape."""
     lz = max(p.Lz for p in params)
     if params[0].advection:
         shapes = [(0, 8)]        # the second-order advection runs at 8-row tiles only
@@ -47,7 +48,7 @@ def candidates(params: list[Params]):
         shapes = [(0, ty) for ty in TILE_Y]
         if all(p.Lx % 2 == 0 for p in params):
             shapes.append((1, 16))
-    return [(k, ty, zc) for k, ty in shapes for zc in Z_CHUNKS if zc <= lz]
+    return [(k, ty, zc) for k, ty in shapes for zc in Z_CHUNKS if zc <= lz] + [(2, 8, 0)]
 
 
 def tune(params: Params | list[Params], steps: int = 12, cache: str | None = CACHE, device=None,

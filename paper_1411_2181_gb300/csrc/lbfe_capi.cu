@@ -88,7 +88,7 @@ lbfe_status derive(const lbfe_params &p, Derived &d) {
 
 struct Layout {
     size_t inst_off, tile_off, item_off, status_off, maps_off;
-    std::vector<size_t> f_off[2], C_off[2], scratch_off, prof_off, mpart_off, dens_off;
+    std::vector<size_t> f_off[2], C_off[2], scratch_off, prof_off, mpart_off, dens_off, pass_off;
     size_t total;
 };
 
@@ -121,6 +121,7 @@ Layout plan(const lbfe_params *p, int n) {
         // reduced storage forms: per-cell offset densities, ping-pong
         L.dens_off.push_back(p[0].precision == LBFE_FP32 ? 0 : take(sizeof(float) * 2 * 2 * S));
     }
+    for (int k = 0; k < n; ++k) L.pass_off.push_back(take(sizeof(unsigned) * (3 * (size_t)p[k].Lz + 1)));
     L.total = off;
     return L;
 }
@@ -146,6 +147,8 @@ struct lbfe_handle {
     int total_items = 0, fused_grid = 0, tile_y = 16, z_chunk_req = 0, num_sms = 0, blocks_per_sm = 0;
     int step_kernel = LBFE_STEP_CELL;
     int advection = 0;               // lbfe_params::advection of every instance
+    bool passes_tuned = false;       // ... because lbfe_tune said so
+    bool passes = false;             // the step runs in three passes (lbfe_passes.cu), else in tiles
     unsigned inject = 0;             // lbfe_test_inject bits
     unsigned *status = nullptr;
     int cur = 0;
@@ -183,6 +186,8 @@ struct lbfe_handle {
         c.tile_y = tile_y;
         c.step_kernel = step_kernel;
         c.advection = advection;
+        c.num_sms = num_sms;
+        c.lost_counts = (inject & LBFE_INJECT_LOST_COUNTS) != 0;
         return c;
     }
 };
@@ -281,6 +286,47 @@ static lbfe_status configure_fused(lbfe_handle *h, int step_kernel, int tile_y, 
     if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
     if (e != cudaSuccess) return cuda_fail(e, "configure_fused");
     return LBFE_OK;
+}
+
+// The three-pass step needs the tensor maps of every instance's runs.
+static bool passes_possible(const lbfe_handle *h) {
+    for (auto &m : h->maps)
+        if (!m.runs_ok) return false;
+    if (lbfe::passes_prepare(h->precision, h->advection) == cudaSuccess) return true;
+    cudaGetLastError();              // not available on this device: the tiles are
+    return false;
+}
+
+// Whether a new handle's steps run in three passes instead of tiles: the
+// smaller estimate of a step's time (the fields are the same bit for bit).
+//   tiles   planes that the busiest block marches, 3.2 us each (8 rows, FP32),
+//           4.4 (12 rows, 2-byte storage), 3.7 (second-order advection), half
+//           as much again where rows are no 16-byte multiples (no copies);
+//   passes  about 11 us of launch and dependent passes, then 0.105 ns a cell
+//           (FP32), 0.117 (FP16), 0.127 (BF16), 0.19 (second-order advection).
+// Measured, us per step, tiles / passes (GB300, FP32 unless noted): 32^3
+// 37 / 15, 37^3 41 / 17, 240 x 20 x 17 41 / 21, 96 x 48 x 48 39 / 35, 64^3
+// 39 / 42, 141 x 75 x 53 104 / 70 (FP16 103 / 81), 40 x 128 x 90 144 / 57,
+// 100 x 96 x 80 111 / 84 (FP16 221 / 93), 192 x 96 x 80 142 / 162 (FP16 141 /
+// 178, second order 164 / 303), 256 x 128 x 64 211 / 238, sixteen 320 x 44 x 40
+// 1107 / 960 (FP16 934 / 1061).
+static bool prefer_passes(const lbfe_handle *h) {
+    const bool fp32 = h->precision == LBFE_FP32;
+    double planes = 0.0, most = 0.0, cells = 0.0;
+    for (int k = 0; k < h->n; ++k) {
+        const InstDev &I = h->inst[k];
+        const double w = h->maps[k].ok ? 1.0 : 1.5;
+        planes += w * I.ntx * I.nty * (I.Lz + 4.0 * I.nzc);
+        most = std::max(most, w * (I.zc + 4.0));
+        cells += (double)I.N;
+    }
+    const double slots = (double)h->num_sms * h->blocks_per_sm;
+    double march = most;
+    if (h->total_items > slots)
+        march = h->n == 1 ? most * std::ceil(h->total_items / slots) : planes / slots + most;
+    const double tile = march * (h->advection ? 3.7 : (fp32 ? 3.2 : 4.4));
+    const double ns = h->advection ? 0.19 : (fp32 ? 0.105 : (h->precision == LBFE_FP16_OFFSET ? 0.117 : 0.127));
+    return 11.0 + 1e-3 * ns * cells < tile;
 }
 
 extern "C" {
@@ -390,6 +436,7 @@ lbfe_status lbfe_create(lbfe_handle **hp, const lbfe_params *p, int n, void *dev
         I.status = h->status + 4 + k;
         I.step_ctr = h->status + 4 + n + 2 * k;
         I.mpart = (double *)(h->base + L.mpart_off[k]);
+        I.pass_cnt = (unsigned *)(h->base + L.pass_off[k]);
         I.G = (float)p[k].G;
         I.Uw = (float)p[k].Uw;
         I.nu_A = (float)d.nu_A;
@@ -411,6 +458,7 @@ lbfe_status lbfe_create(lbfe_handle **hp, const lbfe_params *p, int n, void *dev
     cudaError_t e = cudaMemcpyAsync(h->inst_dev, h->inst.data(), sizeof(InstDev) * n, cudaMemcpyHostToDevice, h->stream);
     if (e == cudaSuccess) e = cudaMemcpyAsync(h->tile_off, toff.data(), sizeof(int) * (n + 1), cudaMemcpyHostToDevice, h->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(h->status, 0, sizeof(unsigned) * (4 + 3 * (size_t)n), h->stream);
+    if (e == cudaSuccess) e = cudaMemsetAsync(h->base + L.pass_off[0], 0, L.total - L.pass_off[0], h->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
     int dev = 0;
     if (e == cudaSuccess) e = cudaGetDevice(&dev);
@@ -427,6 +475,7 @@ lbfe_status lbfe_create(lbfe_handle **hp, const lbfe_params *p, int n, void *dev
         delete h;
         return st;
     }
+    h->passes = passes_possible(h) && prefer_passes(h);
     *hp = h;
     return LBFE_OK;
 }
@@ -477,6 +526,16 @@ lbfe_status lbfe_step(lbfe_handle *h, long long nsteps) {
     CK(cudaStreamIsCapturing(h->stream, &cs));
     const bool graphs = nsteps >= 2 && cs == cudaStreamCaptureStatusNone;
     const lbfe::LaunchCtx c = h->ctx();
+    if (h->passes && !(h->inject & LBFE_INJECT_SHORT_COPIES)) {
+        for (long long t = 0; t < nsteps;) {
+            const int m = (int)std::min<long long>(lbfe::passes_steps(), nsteps - t);
+            CK(lbfe::launch_passes(c, h->cur, m));
+            if (m & 1) h->cur ^= 1;
+            t += m;
+        }
+        for (int k = 0; k < h->n; ++k) h->steps[k] += nsteps;
+        return LBFE_OK;
+    }
     for (long long t = 0; t < nsteps; ++t) {
         if (graphs) {
             if (!h->step_graph[h->cur]) CK(build_step_graph(h, h->cur));
@@ -676,7 +735,7 @@ lbfe_status lbfe_set_columns(lbfe_handle *h, int k, int x0, int nx, const void *
 }
 
 lbfe_status lbfe_test_inject(lbfe_handle *h, unsigned what) {
-    if (!h || (what & ~(unsigned)LBFE_INJECT_SHORT_COPIES)) return LBFE_ERR_BAD_PARAM;
+    if (!h || (what & ~(unsigned)(LBFE_INJECT_SHORT_COPIES | LBFE_INJECT_LOST_COUNTS))) return LBFE_ERR_BAD_PARAM;
     CK(cudaStreamSynchronize(h->stream));
     h->inject = what;
     // rebuild the tensor maps of the current launch shape
@@ -685,13 +744,21 @@ lbfe_status lbfe_test_inject(lbfe_handle *h, unsigned what) {
 
 lbfe_status lbfe_tune(lbfe_handle *h, int step_kernel, int tile_y, int z_chunk) {
     if (!h) return LBFE_ERR_BAD_PARAM;
-    return configure_fused(h, step_kernel, tile_y, z_chunk);
+    if (step_kernel == LBFE_STEP_PASSES) {
+        if (tile_y != 8 || z_chunk != 0 || !passes_possible(h)) return LBFE_ERR_BAD_PARAM;
+        CK(cudaStreamSynchronize(h->stream));
+        h->passes = h->passes_tuned = true;
+        return LBFE_OK;
+    }
+    const lbfe_status st = configure_fused(h, step_kernel, tile_y, z_chunk);
+    if (st == LBFE_OK) h->passes = h->passes_tuned = false;
+    return st;
 }
 
 lbfe_status lbfe_launch_config(const lbfe_handle *h, int *step_kernel, int *tile_y, int *z_chunk, int *grid,
                                int *items) {
     if (!h) return LBFE_ERR_BAD_PARAM;
-    if (step_kernel) *step_kernel = h->step_kernel;
+    if (step_kernel) *step_kernel = h->passes_tuned ? LBFE_STEP_PASSES : h->step_kernel;
     if (tile_y) *tile_y = h->tile_y;
     if (z_chunk) *z_chunk = h->inst[0].zc;
     if (grid) *grid = h->fused_grid;

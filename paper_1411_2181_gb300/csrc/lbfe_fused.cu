@@ -519,12 +519,21 @@ int fused_launches(int n) { return n <= 1 ? 1 : (n + kStepMaxInst - 1) / kStepMa
 cudaError_t fused_pop_maps(const InstDev &I, int precision, int tile_y, bool short_box, PopMaps *m) {
     std::memset(m, 0, sizeof *m);
     const size_t esz = precision == LBFE_FP32 ? 4 : 2;
-    if (((size_t)I.Lx * esz) % 16 != 0 || ((size_t)I.Lx * 4) % 16 != 0) return cudaSuccess;
     EncodeTiledFn fn = encode_tiled();
     if (!fn) return cudaSuccess;
     const CUtensorMapDataType dt = precision == LBFE_FP16_OFFSET   ? CU_TENSOR_MAP_DATA_TYPE_FLOAT16
                                    : precision == LBFE_BF16_OFFSET ? CU_TENSOR_MAP_DATA_TYPE_BFLOAT16
                                                                    : CU_TENSOR_MAP_DATA_TYPE_FLOAT32;
+    // the three-pass step's runs: any extents (S is a multiple of 64 elements)
+    m->runs_ok = 1;
+    for (int b = 0; b < 2; ++b) {
+        const cuuint64_t d[2] = {(cuuint64_t)I.S, (cuuint64_t)(2 * Q)}, st[1] = {(cuuint64_t)I.S * esz};
+        const cuuint32_t bx[2] = {256u, (cuuint32_t)(2 * Q)}, es[2] = {1u, 1u};
+        if (fn(&m->m[b].runs, dt, 2, I.f[b], d, st, bx, es, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
+               CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
+            m->runs_ok = 0;
+    }
+    if (((size_t)I.Lx * esz) % 16 != 0 || ((size_t)I.Lx * 4) % 16 != 0) return cudaSuccess;
     const bool region = tile_y <= 12;
     const cuuint32_t xpad = (cuuint32_t)(16 / esz), ty = (cuuint32_t)tile_y;
     const cuuint64_t dims[4] = {(cuuint64_t)I.Lx, (cuuint64_t)I.Ly, (cuuint64_t)I.Lz, (cuuint64_t)(2 * Q)};
@@ -552,7 +561,6 @@ cudaError_t fused_pop_maps(const InstDev &I, int precision, int tile_y, bool sho
         if (r == CUDA_SUCCESS && region && esz == 2 && I.dens[b ^ 1])
             r = enc(&sm.dens, CU_TENSOR_MAP_DATA_TYPE_INT64, 3, I.dens[b ^ 1], ddims, dstrides, dbox);
         if (r != CUDA_SUCCESS) {
-            std::memset(m, 0, sizeof *m);
             return cudaSuccess;
         }
     }

@@ -113,6 +113,7 @@ struct InstDev {
     int ntx, nty, nzc, zc;           // fused kernel: column tiles in x, y; z-chunks and their depth
     unsigned *status;                // this instance's status word (may be null)
     unsigned *step_ctr;              // time steps taken, [2] by ping-pong parity (BF16 rounding seed)
+    unsigned *pass_cnt;              // three-pass step: finished cells [3][Lz] by pass and plane, their value at launch
 };
 
 // Raise a status flag for the whole launch and, when present, for instance I.
@@ -182,6 +183,8 @@ struct LaunchCtx {
     int step_kernel;                 // lbfe_step_kernel
     int advection = 0;               // lbfe_params::advection of the batch
     int fused_slots;                 // resident blocks of the fused kernel on the GPU
+    int num_sms = 0;
+    int lost_counts = 0;             // test hook of the three-pass step
     const struct PopMaps *maps_host; // per instance: TMA maps of the step kernel (may be null)
     const struct StepMaps *maps_dev; // device copies, [instance][parity]
 };
@@ -193,17 +196,23 @@ struct StepMaps {
     CUtensorMap pop;    // box of the tile's own cells (16 rows) or of its radius-2 region (8, 12 rows)
     CUtensorMap c;      // conformation, region box
     CUtensorMap dens;   // offset densities (float2 per cell), region box
+    CUtensorMap runs;   // populations as [38][S], box of 256 cells (three-pass step)
 };
 // Both parities of an instance; ok = 0 when the instance's layout does not
-// allow TMA (the kernel then reads with ordinary loads).
+// allow TMA (the tile kernels then read with ordinary loads).
 struct PopMaps {
     StepMaps m[2];
-    int ok;
+    int ok;             // pop, c, dens
+    int runs_ok;
 };
 // short_box (test hook): population boxes one row short of what the step
 // kernel expects, so that its waits for them expire
 cudaError_t fused_pop_maps(const InstDev &I, int precision, int tile_y, bool short_box, PopMaps *m);
 cudaError_t launch_fused(const LaunchCtx &c, int cur);
+// The three-pass step (lbfe_passes.cu): up to passes_steps() steps in a launch.
+cudaError_t launch_passes(const LaunchCtx &c, int cur, int steps);
+cudaError_t passes_prepare(int precision, int advection);
+int passes_steps();
 // Kernel launches of one time step of n instances.
 int fused_launches(int n);
 // Resident blocks per SM of the fused kernel for a tile height.

@@ -25,8 +25,8 @@ if not os.path.exists(LIB_PATH):
 _lib = ct.CDLL(LIB_PATH)
 
 FIELD_F, FIELD_C, FIELD_RHO, FIELD_U = 0, 1, 2, 3
-STEP_CELL, STEP_PAIR = 0, 1   # lbfe_step_kernel
-INJECT_SHORT_COPIES = 1       # lbfe_test_inject
+STEP_CELL, STEP_PAIR, STEP_PASSES = 0, 1, 2        # lbfe_step_kernel
+INJECT_SHORT_COPIES, INJECT_LOST_COUNTS = 1, 2     # lbfe_test_inject
 
 OK, ERR_BAD_PARAM, ERR_NO_MEMORY, ERR_CUDA, ERR_DIVERGED, ERR_TIMEOUT, ERR_STATE, ERR_IO = range(8)
 
@@ -210,7 +210,8 @@ class Solver:
 
     def tune(self, tile_y: int = 8, z_chunk: int = 0, kernel: int = 0):
         """Launch shape of the step: kernel STEP_CELL (tile_y in 8, 12, 16) or
-        STEP_PAIR (tile_y 16, even Lx), and the z-chunk depth (0 = auto)."""
+        STEP_PAIR (tile_y 16, even Lx), and the z-chunk depth (0 = auto), or
+        STEP_PASSES (tile_y 8, z_chunk 0)."""
         _check(_lib.lbfe_tune(self._h, int(kernel), int(tile_y), int(z_chunk)), "lbfe_tune")
 
     def launch_config(self) -> dict:

@@ -128,12 +128,11 @@ def run_batch(cases: list[Case], device=None, stats: dict | None = None) -> list
     t0 = time.perf_counter()
     with torch.cuda.stream(stream):
         s = lbfe.Solver(ps, device=device, stream=stream)
-        # one launch shape for every batch: the 8-row one-cell kernel (the
-        # fastest FP32 shape), z-chunks fitted to the batch.  The z-chunk
-        # does not change a cell's arithmetic, the kernel variant and tile
-        # height can (FP32 rounding), and a verdict near the threshold must
-        # not depend on which batch the case ran in
-        s.tune(8, 0, 0)
+        # the launch shape a new handle takes: 8-row tiles with z-chunks fitted
+        # to the batch, or the three-pass kernel where that is faster.  Neither
+        # the z-chunk nor that choice changes a cell's arithmetic (the other
+        # variants can, by FP32 rounding), and a verdict near the threshold
+        # must not depend on which batch the case ran in
         for k, (c, p) in enumerate(zip(cases, ps)):
             s.init(k, synth.droplet_densities(p.Lx, p.Ly, p.Lz, p.R, p.rho_in, p.rho_out, 1e-4, seed=c.seed))
         n = len(cases)
@@ -203,7 +202,6 @@ def breakup_details(cases: list[Case], device=None, every_tem: float = 0.25, aft
     stream = torch.cuda.Stream(device)
     with torch.cuda.stream(stream):
         s = lbfe.Solver(ps, device=device, stream=stream)
-        s.tune(8, 0, 0)
         for k, (c, p) in enumerate(zip(cases, ps)):
             s.init(k, synth.droplet_densities(p.Lx, p.Ly, p.Lz, p.R, p.rho_in, p.rho_out, 1e-4, seed=c.seed))
         nxt, steps = list(every), 0
