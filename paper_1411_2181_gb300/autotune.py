@@ -36,11 +36,14 @@ def _load(path):
         return {}
 
 
+# the three-pass kernel has one shape, tried beside the tile shapes
+PASSES = (2, 8, 0)
+
+
 def candidates(params: list[Params]):
     """(kernel, tile_y, z_chunk) triples: cell kernel (0) at every tile
     height, pair kernel (1) at 16 rows when every Lx is even; with the
-    second-order advection scheme the cell kernel at 8 rows only.  The
-    three-pass kernel (2) has one shape."""
+    second-order advection scheme the cell kernel at 8 rows only."""
     lz = max(p.Lz for p in params)
     if params[0].advection:
         shapes = [(0, 8)]        # the second-order advection runs at 8-row tiles only
@@ -48,7 +51,7 @@ def candidates(params: list[Params]):
         shapes = [(0, ty) for ty in TILE_Y]
         if all(p.Lx % 2 == 0 for p in params):
             shapes.append((1, 16))
-    return [(k, ty, zc) for k, ty in shapes for zc in Z_CHUNKS if zc <= lz] + [(2, 8, 0)]
+    return [(k, ty, zc) for k, ty in shapes for zc in Z_CHUNKS if zc <= lz]
 
 
 def tune(params: Params | list[Params], steps: int = 12, cache: str | None = CACHE, device=None,
@@ -73,7 +76,7 @@ def tune(params: Params | list[Params], steps: int = 12, cache: str | None = CAC
                                                          np.full((p.Lz, p.Ly, p.Lx), p.rho_out)])
             s.init(k, r)
         trials = []
-        for kern, ty, zc in candidates(plist):
+        for kern, ty, zc in candidates(plist) + [PASSES]:
             s.tune(ty, zc, kern)
             s.step(2)
             e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
