@@ -71,6 +71,16 @@ lbfe_status lbfe_mlp_get_grads(lbfe_mlp *m, float *host_grads);
  * w -= lr (m/(1-b1^t) / (sqrt(v/(1-b2^t)) + eps) + wd w). */
 lbfe_status lbfe_mlp_adamw(lbfe_mlp *m, float lr, float beta1, float beta2, float eps, float weight_decay);
 
+/* One epoch of mini-batch training on consecutive rows: for each batch of up to
+ * `batch` of the `rows` rows, the gradient as by lbfe_mlp_loss_grad and one
+ * step as by lbfe_mlp_adamw (the same results), without a host synchronisation
+ * between the batches.  loss_sum_host (may be NULL) receives the sum over the
+ * batches of their loss times their rows; with it the call synchronises the
+ * stream at its end.  1 <= batch <= max_batch, rows >= 1. */
+lbfe_status lbfe_mlp_epoch(lbfe_mlp *m, const float *x_dev, const float *t_dev, const float *mask_dev, int rows,
+                           int batch, float lr, float beta1, float beta2, float eps, float weight_decay,
+                           double *loss_sum_host);
+
 lbfe_status lbfe_mlp_destroy(lbfe_mlp *m);
 
 #ifdef __cplusplus

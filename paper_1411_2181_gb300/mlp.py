@@ -24,9 +24,12 @@ _lib.lbfe_mlp_forward.argtypes = [_M, ct.c_void_p, ct.c_int, ct.c_void_p]
 _lib.lbfe_mlp_loss_grad.argtypes = [_M, ct.c_void_p, ct.c_void_p, ct.c_void_p, ct.c_int, _F]
 _lib.lbfe_mlp_get_grads.argtypes = [_M, _F]
 _lib.lbfe_mlp_adamw.argtypes = [_M, ct.c_float, ct.c_float, ct.c_float, ct.c_float, ct.c_float]
+_lib.lbfe_mlp_epoch.argtypes = ([_M] + [ct.c_void_p] * 3 + [ct.c_int] * 2 + [ct.c_float] * 5 +
+                                [ct.POINTER(ct.c_double)])
 _lib.lbfe_mlp_destroy.argtypes = [_M]
 for _fn in ("lbfe_mlp_required_bytes", "lbfe_mlp_create", "lbfe_mlp_set_params", "lbfe_mlp_get_params",
-            "lbfe_mlp_forward", "lbfe_mlp_loss_grad", "lbfe_mlp_get_grads", "lbfe_mlp_adamw", "lbfe_mlp_destroy"):
+            "lbfe_mlp_forward", "lbfe_mlp_loss_grad", "lbfe_mlp_get_grads", "lbfe_mlp_adamw", "lbfe_mlp_epoch",
+            "lbfe_mlp_destroy"):
     getattr(_lib, _fn).restype = ct.c_int
 
 DIMS = (6, 128, 128, 128, 128, 4)
@@ -129,19 +132,14 @@ class MLP:
         for ep in range(epochs):
             perm = torch.as_tensor(rng.permutation(n), device=self.device)
             lr_e = lr_final + 0.5 * (lr - lr_final) * (1 + np.cos(np.pi * ep / max(1, epochs - 1)))
-            tot = 0.0
-            for s in range(0, n, bs):
-                idx = perm[s:s + bs]
-                xb, tb, mb = Xd[idx].contiguous(), Td[idx].contiguous(), Md[idx].contiguous()
-                torch.cuda.synchronize(self.device)
-                loss = ct.c_float()
-                _check(_lib.lbfe_mlp_loss_grad(self._h, ct.c_void_p(xb.data_ptr()), ct.c_void_p(tb.data_ptr()),
-                                               ct.c_void_p(mb.data_ptr()), xb.shape[0], ct.byref(loss)),
-                       "lbfe_mlp_loss_grad")
-                _check(_lib.lbfe_mlp_adamw(self._h, float(lr_e), 0.9, 0.999, 1e-8, float(weight_decay)),
-                       "lbfe_mlp_adamw")
-                tot += loss.value * xb.shape[0]
-            hist.append(tot / n)
+            # the epoch's rows in its order, then every mini-batch in one call
+            xb, tb, mb = Xd[perm], Td[perm], Md[perm]
+            torch.cuda.synchronize(self.device)
+            tot = ct.c_double()
+            _check(_lib.lbfe_mlp_epoch(self._h, ct.c_void_p(xb.data_ptr()), ct.c_void_p(tb.data_ptr()),
+                                       ct.c_void_p(mb.data_ptr()), n, bs, float(lr_e), 0.9, 0.999, 1e-8,
+                                       float(weight_decay), ct.byref(tot)), "lbfe_mlp_epoch")
+            hist.append(tot.value / n)
             if verbose and ep % max(1, epochs // 10) == 0:
                 print(f"epoch {ep} loss {hist[-1]:.5f}")
         return hist

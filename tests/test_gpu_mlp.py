@@ -121,3 +121,32 @@ def test_row_blocks_and_batch_parts(M, B, bf16):
     assert per_tensor_err(g, gr) < TOL_CHAIN
     assert net.loss_grad(x, t, mask) == loss and np.array_equal(net.grads(), g)
     assert np.array_equal(net.forward(x), y)
+
+
+@pytest.mark.parametrize("bf16", [False, True])
+@pytest.mark.parametrize("n,bs", [(1, 1), (37, 37), (300, 64), (130, 65)])
+def test_epoch_equals_single_steps(M, n, bs, bf16):
+    """An epoch in one call gives the bits of its mini-batches one by one
+    (gradient, then step): parameters, last gradient and loss."""
+    import ctypes as ct
+    import torch
+    p = M.init_params(n)
+    x, t, mask = batch(n, n + 2)
+    a, b = M.MLP(max_batch=bs, bf16=bf16), M.MLP(max_batch=bs, bf16=bf16)
+    a.set_params(p)
+    b.set_params(p)
+    d = [torch.from_numpy(v).cuda() for v in (x, t, mask)]
+    torch.cuda.synchronize()
+    for _ in range(2):
+        tot = ct.c_double()
+        assert M._lib.lbfe_mlp_epoch(a._h, *[ct.c_void_p(v.data_ptr()) for v in d], n, bs, 1e-3, 0.9, 0.999, 1e-8, 1e-2,
+                                     ct.byref(tot)) == 0
+        want = 0.0
+        for s in range(0, n, bs):
+            e = slice(s, s + bs)
+            want += b.loss_grad(x[e], t[e], mask[e]) * len(x[e])
+            b.adamw(lr=1e-3, weight_decay=1e-2)
+        assert tot.value == want
+        assert np.array_equal(a.get_params(), b.get_params()) and np.array_equal(a.grads(), b.grads())
+    assert M._lib.lbfe_mlp_epoch(a._h, *[ct.c_void_p(v.data_ptr()) for v in d], n, bs + 1, 1e-3, 0.9, 0.999, 1e-8, 0.0,
+                                 None) != 0
