@@ -124,7 +124,7 @@ __device__ __forceinline__ void raise_flag(unsigned *global, const InstDev &I, u
 
 constexpr int kBlock = 256;          // threads per block of the cell-per-thread kernels
 constexpr int kMaxLx = 4096;         // largest Lx lbfe_derive accepts
-constexpr int kObsBlocks = 608;      // 4 x 152 SMs for the observables reduction
+constexpr int kObsBlocks = 456;      // observables reduction: the three blocks of an SM that 75 registers leave
 static_assert(kObsBlocks >= (kMaxLx + 31) / 32, "a block per 32 x-planes");
 // Observables record: 6 Lx plane sums, the masses, the status word, a counter.
 __host__ __device__ constexpr size_t obs_words(int Lx) { return 6 * (size_t)Lx + 4; }
