@@ -292,41 +292,46 @@ static lbfe_status configure_fused(lbfe_handle *h, int step_kernel, int tile_y, 
 static bool passes_possible(const lbfe_handle *h) {
     for (auto &m : h->maps)
         if (!m.runs_ok) return false;
-    if (lbfe::passes_prepare(h->precision, h->advection) == cudaSuccess) return true;
+    if (lbfe::passes_prepare(h->n, h->precision, h->advection) == cudaSuccess) return true;
     cudaGetLastError();              // not available on this device: the tiles are
     return false;
 }
 
 // Whether a new handle's steps run in three passes instead of tiles: the
 // smaller estimate of a step's time (the fields are the same bit for bit).
-//   tiles   planes that the busiest block marches, 3.2 us each (8 rows, FP32),
-//           4.4 (12 rows, 2-byte storage), 3.7 (second-order advection), half
-//           as much again where rows are no 16-byte multiples (no copies);
-//   passes  about 11 us of launch and dependent passes, then 0.105 ns a cell
-//           (FP32), 0.117 (FP16), 0.127 (BF16), 0.19 (second-order advection).
+//   tiles   planes that the busiest block marches, 3.2 us each (8 rows, FP32;
+//           3.6 in batches), 4.4 (12 rows, 2-byte storage), 3.7 (second-order
+//           advection), half as much again where rows are no 16-byte
+//           multiples (no copies);
+//   passes  about 8 us of launch and dependent passes, 0.5 ns a cell of the
+//           largest plane (a pass stays two planes behind the one before) and
+//           0.100 ns a cell (FP32), 0.105 (FP16), 0.112 (BF16), 0.15
+//           (second-order advection), a tenth more in batches.
 // Measured, us per step, tiles / passes (GB300, FP32 unless noted): 32^3
-// 37 / 15, 37^3 41 / 17, 240 x 20 x 17 41 / 21, 96 x 48 x 48 39 / 35, 64^3
-// 39 / 42, 141 x 75 x 53 104 / 70 (FP16 103 / 81), 40 x 128 x 90 144 / 57,
-// 100 x 96 x 80 111 / 84 (FP16 221 / 93), 192 x 96 x 80 142 / 162 (FP16 141 /
-// 178, second order 164 / 303), 256 x 128 x 64 211 / 238, sixteen 320 x 44 x 40
-// 1107 / 960 (FP16 934 / 1061).
+// 35 / 15, 37^3 41 / 17, 240 x 20 x 17 41 / 21, 96 x 48 x 48 39 / 30, 64^3
+// 37 / 32 (FP16 51 / 45), 141 x 75 x 53 103 / 62 (FP16 101 / 75), 40 x 128 x 90
+// 94 / 53, 128 x 128 x 16 37 / 41, 100 x 96 x 80 109 / 83 (FP16 141 / 87), 192 x 96 x 80 142 / 160
+// (FP16 140 / 165, BF16 145 / 175, second order 160 / 233), 256 x 128 x 64
+// 212 / 235, sixteen 320 x 44 x 40 1024 / 972 (FP16 853 / 1076),
+// twelve uneven lattices 2345 / 1987 (FP16 1874 / 2074).
 static bool prefer_passes(const lbfe_handle *h) {
     const bool fp32 = h->precision == LBFE_FP32;
-    double planes = 0.0, most = 0.0, cells = 0.0;
+    double planes = 0.0, most = 0.0, cells = 0.0, plane = 0.0;
     for (int k = 0; k < h->n; ++k) {
         const InstDev &I = h->inst[k];
         const double w = h->maps[k].ok ? 1.0 : 1.5;
         planes += w * I.ntx * I.nty * (I.Lz + 4.0 * I.nzc);
         most = std::max(most, w * (I.zc + 4.0));
         cells += (double)I.N;
+        plane = std::max(plane, (double)I.Lx * I.Ly);
     }
     const double slots = (double)h->num_sms * h->blocks_per_sm;
     double march = most;
     if (h->total_items > slots)
         march = h->n == 1 ? most * std::ceil(h->total_items / slots) : planes / slots + most;
-    const double tile = march * (h->advection ? 3.7 : (fp32 ? 3.2 : 4.4));
-    const double ns = h->advection ? 0.19 : (fp32 ? 0.105 : (h->precision == LBFE_FP16_OFFSET ? 0.117 : 0.127));
-    return 11.0 + 1e-3 * ns * cells < tile;
+    const double tile = march * (h->advection ? 3.7 : (fp32 ? (h->n > 1 ? 3.6 : 3.2) : 4.4));
+    const double ns = h->advection ? 0.15 : (fp32 ? 0.100 : (h->precision == LBFE_FP16_OFFSET ? 0.105 : 0.112));
+    return 8.0 + 0.5e-3 * plane + 1e-3 * ns * (h->n > 1 ? 1.1 : 1.0) * cells < tile;
 }
 
 extern "C" {

@@ -211,7 +211,7 @@ cudaError_t fused_pop_maps(const InstDev &I, int precision, int tile_y, bool sho
 cudaError_t launch_fused(const LaunchCtx &c, int cur);
 // The three-pass step (lbfe_passes.cu): up to passes_steps() steps in a launch.
 cudaError_t launch_passes(const LaunchCtx &c, int cur, int steps);
-cudaError_t passes_prepare(int precision, int advection);
+cudaError_t passes_prepare(int n, int precision, int advection);
 int passes_steps();
 // Kernel launches of one time step of n instances.
 int fused_launches(int n);

@@ -15,8 +15,8 @@
 // lattice of few columns still fills the GPU.  They pay with the populations'
 // second read (the L2 serves part of it), 40 bytes a cell of scratch and more
 // instructions.  Measured in FP32, tile kernel -> passes, us per step: 32^3
-// 35 -> 15, 141 x 75 x 53 103 -> 71, sixteen 320 x 44 x 40 1107 -> 970;
-// 192 x 96 x 80 142 -> 164 (the tile kernel stays).
+// 35 -> 15, 64^3 37 -> 32, 141 x 75 x 53 103 -> 62, sixteen 320 x 44 x 40
+// 1107 -> 970; 192 x 96 x 80 142 -> 160 (the tile kernel stays).
 // Which of the two a handle runs is decided in lbfe_capi.cu (prefer_passes).
 //
 // Work.  A slot is one pass over up to R x 256 cells.  Slots are numbered so
@@ -40,8 +40,8 @@
 // hide behind the stencils' and behind the wait of the next slot.  With the
 // populations in registers (38 ordinary loads ahead of the stencil) the
 // 192 x 96 x 80 step took 186 us, with staging 166, with the scheduling warp
-// 160, with the L2 hints of the copies 154 (with packed stencil sums; 164 with
-// the tile kernels' sums, which keep the bits).
+// 160, with the L2 hints of the copies 154 (with packed stencil sums; 160 with
+// the tile kernels' sums, which keep the bits, and ONE).
 // Bound by latency at sixteen computing warps of 104 or 112 registers (issue
 // slots 38 % busy) and, on large lattices, DRAM (about 530 bytes a cell).
 #include <type_traits>
@@ -462,7 +462,10 @@ constexpr int pass_smem() {
     return kTeams * 2 * 2 * Q * kRun * (int)sizeof(T) + 128;
 }
 
-template <typename T, bool ADV2>
+// ONE: a launch of one instance, whose descriptor's address is then a constant
+// (base addresses in uniform registers: 192 x 96 x 80 164 -> 160 us in FP32,
+// 180 -> 165 in FP16).
+template <typename T, bool ADV2, bool ONE>
 __global__ void __launch_bounds__(kPassThreads, 1) k_passes(const __grid_constant__ PassArgs A) {
     __shared__ Job t_job[kTeams][2], t_cur[kTeams];   // handed over; worked on
     // per team, two of each: run copied, run read, job known, job read
@@ -521,7 +524,7 @@ __global__ void __launch_bounds__(kPassThreads, 1) k_passes(const __grid_constan
                     const int mid = (k + hi + 1) >> 1;
                     if (A.item_off[mid] <= item) k = mid; else hi = mid - 1;
                 }
-                const PassInst &I = A.inst[k];
+                const PassInst &I = A.inst[ONE ? 0 : k];
                 const int Lz = I.Lz;
                 const u32 c0 = (u32)(item - A.item_off[k]) * cells, c1 = min(c0 + cells, I.N);
                 // the pass before on the slot's planes and the ones beside them;
@@ -601,7 +604,7 @@ __global__ void __launch_bounds__(kPassThreads, 1) k_passes(const __grid_constan
         const Job J = t_cur[team];
         const int pass = J.pass, b = (A.parity + J.step) & 1;
         if (pass == kPassEnd) break;
-        const PassInst &I = A.inst[J.k];
+        const PassInst &I = A.inst[ONE ? 0 : J.k];
         const u32 c0 = J.c0, c1 = J.c1;
         if (pass < 2) {
             unsigned seed = 0;
@@ -668,26 +671,36 @@ void fast_div(u32 d, u32 &mul, unsigned char &sh) {
     sh = (unsigned char)((l > 0 ? 0x80 : 0) | (l > 0 ? l - 1 : 0));
 }
 
-template <typename T, bool ADV2>
-cudaError_t passes_t(const PassArgs *a, int grid, cudaStream_t st) {
+template <typename T, bool ADV2, bool ONE>
+cudaError_t passes_k(const PassArgs *a, int grid, cudaStream_t st) {
     if (!a)   // prepare
-        return cudaFuncSetAttribute(k_passes<T, ADV2>, cudaFuncAttributeMaxDynamicSharedMemorySize, pass_smem<T>());
-    k_passes<T, ADV2><<<grid, kPassThreads, pass_smem<T>(), st>>>(*a);
+        return cudaFuncSetAttribute(k_passes<T, ADV2, ONE>, cudaFuncAttributeMaxDynamicSharedMemorySize, pass_smem<T>());
+    k_passes<T, ADV2, ONE><<<grid, kPassThreads, pass_smem<T>(), st>>>(*a);
     return cudaGetLastError();
 }
 
-cudaError_t passes_form(const PassArgs *a, int precision, int advection, int grid, cudaStream_t st) {
+template <typename T, bool ADV2>
+cudaError_t passes_t(const PassArgs *a, int n, int grid, cudaStream_t st) {
+    return n == 1 ? passes_k<T, ADV2, true>(a, grid, st) : passes_k<T, ADV2, false>(a, grid, st);
+}
+
+cudaError_t passes_form(const PassArgs *a, int n, int precision, int advection, int grid, cudaStream_t st) {
     switch (precision) {
-        case LBFE_FP16_OFFSET: return advection ? passes_t<__half, true>(a, grid, st) : passes_t<__half, false>(a, grid, st);
+        case LBFE_FP16_OFFSET: return advection ? passes_t<__half, true>(a, n, grid, st) : passes_t<__half, false>(a, n, grid, st);
         case LBFE_BF16_OFFSET:
-            return advection ? passes_t<__nv_bfloat16, true>(a, grid, st) : passes_t<__nv_bfloat16, false>(a, grid, st);
-        default: return advection ? passes_t<float, true>(a, grid, st) : passes_t<float, false>(a, grid, st);
+            return advection ? passes_t<__nv_bfloat16, true>(a, n, grid, st) : passes_t<__nv_bfloat16, false>(a, n, grid, st);
+        default: return advection ? passes_t<float, true>(a, n, grid, st) : passes_t<float, false>(a, n, grid, st);
     }
 }
 
 }  // namespace
 
-cudaError_t passes_prepare(int precision, int advection) { return passes_form(nullptr, precision, advection, 0, nullptr); }
+// For launches of n instances (the last group of a larger batch may be one).
+cudaError_t passes_prepare(int n, int precision, int advection) {
+    cudaError_t e = passes_form(nullptr, n, precision, advection, 0, nullptr);
+    if (e == cudaSuccess && n > 1 && n % kStepMaxInst == 1) e = passes_form(nullptr, 1, precision, advection, 0, nullptr);
+    return e;
+}
 
 // Up to kPassSteps steps of every instance from state parity cur: one launch
 // per 64 instances.
@@ -704,9 +717,11 @@ cudaError_t launch_passes(const LaunchCtx &c, int cur, int steps) {
         a.lost = c.lost_counts;
         long long cells = 0;
         for (int k = k0; k < k1; ++k) cells += c.inst_host[k].N;
-        // runs of a slot: as many as leave every team two slots a pass
+        // runs of a slot: as many as leave every team a slot a pass (two slots:
+        // 64^3 41.5 us against 31.8, 141 x 75 x 53 70 against 61.5; half a slot:
+        // 96 x 48 x 48 34.1 against 30.2)
         int R = 1;
-        while (R < kMaxRuns && cells / (kRun * 2 * R) >= 2 * workers) R *= 2;
+        while (R < kMaxRuns && cells / (kRun * 2 * R) >= workers) R *= 2;
         a.R = R;
         const long long ic = (long long)kRun * R;
         long long items = 0;
@@ -763,7 +778,7 @@ cudaError_t launch_passes(const LaunchCtx &c, int cur, int steps) {
         if (slots > 0x3fffffffll) return cudaErrorInvalidValue;
         a.slots = (int)slots;
         const int grid = ((a.slots < workers ? a.slots : workers) + kTeams - 1) / kTeams;
-        const cudaError_t e = passes_form(&a, c.precision, c.advection, grid, c.stream);
+        const cudaError_t e = passes_form(&a, a.n, c.precision, c.advection, grid, c.stream);
         if (e != cudaSuccess) return e;
     }
     return cudaSuccess;
