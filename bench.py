@@ -229,7 +229,7 @@ def measured_peak():
 
 # sources of the step kernels (device code and their launch code); a
 # profile summary stays valid while these are unchanged
-STEP_SOURCES = ("lbfe_internal.cuh", "lbfe_step.cuh", "lbfe_fused.cu", "lbfe_fused2.cu")
+STEP_SOURCES = ("lbfe_internal.cuh", "lbfe_step.cuh", "lbfe_fused.cu", "lbfe_fused2.cu", "lbfe_passes.cu")
 
 
 def kernel_source_hash():
@@ -244,10 +244,11 @@ def kernel_source_hash():
     return h.hexdigest()[:16]
 
 
-def profiled_traffic(workload_name: str, precision: int, advection: int = 0):
+def profiled_traffic(workload_name: str, precision: int, advection: int = 0, kernel: int = 0):
     """DRAM bytes per lattice update of the step from the committed ncu
-    summary, if it was taken on the current kernel sources."""
-    suffix = "_upwind2" if advection else ""
+    summary of the tile kernel or (kernel 2) the three-pass kernel, if it was
+    taken on the current kernel sources."""
+    suffix = ("_upwind2" if advection else "") + ("_passes" if kernel == 2 else "")
     fn = os.path.join(ROOT, "profiles",
                       f"step_{workload_name}_{['fp32', 'fp16', 'bf16'][precision]}{suffix}.md")
     if not os.path.exists(fn):
@@ -357,12 +358,13 @@ def timed_steps(s, stream, steps: int, warmup: int, dist=False):
     return ev0.elapsed_time(ev1)
 
 
-def roofline_record(prec: int, ncell: int, ms_per_step: float, workload_name: str, advection: int):
+def roofline_record(prec: int, ncell: int, ms_per_step: float, workload_name: str, advection: int, kernel: int = 0):
     peak, peak_kind = measured_peak()
     algo = ALGO_BYTES[prec]
     achieved = algo * ncell / (ms_per_step / 1e3) / 1e9
-    traffic_per_lup, prof_file = profiled_traffic(workload_name, prec, advection)
-    return {"bound": "hbm", "kernel": "k_fused (whole time step in one kernel)",
+    traffic_per_lup, prof_file = profiled_traffic(workload_name, prec, advection, kernel)
+    return {"bound": "hbm", "kernel": ("k_passes (three passes in one kernel)" if kernel == 2 else
+                                       "k_fused (whole time step in one kernel)"),
             "achieved": round(achieved, 1), "peak": peak, "peak_kind": peak_kind, "unit": "GB/s",
             "frac": round(achieved / peak, 4), "algorithmic_bytes_per_lup": algo,
             "traffic": (round(traffic_per_lup * ncell) if traffic_per_lup else None),
@@ -391,7 +393,7 @@ def time_form(name: str, prec: int, steps: int, warmup: int, device: str, autotu
     del s
     torch.cuda.empty_cache()
     msps = ms / steps
-    roof = roofline_record(prec, ncell, msps, name, 0)
+    roof = roofline_record(prec, ncell, msps, name, 0, launch["kernel"])
     return {"workload": name, "dtype": DTYPE[prec], "cells": ncell, "steps": steps,
             "value": round(ncell * steps / (ms / 1e3) / 1e6, 2), "unit": METRIC, "ms_per_step": round(msps, 5),
             "roofline": {k: roof[k] for k in ("achieved", "peak", "unit", "frac", "algorithmic_bytes_per_lup",
@@ -479,7 +481,7 @@ def run_ours(a):
                "timed": "lbfe_init (pinned H2D of rho[2][N] float64) + lbfe_step(K) + lbfe_observables"}
     torch.cuda.empty_cache()
 
-    roof = roofline_record(prec, ncell, ms_per_step, a.workload, adv)
+    roof = roofline_record(prec, ncell, ms_per_step, a.workload, adv, launch["kernel"])
 
     # the other forms, each timed on its own (one GPU only: the scaling runs
     # time the headline alone)
