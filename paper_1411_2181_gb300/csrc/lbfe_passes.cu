@@ -476,8 +476,9 @@ __global__ void __launch_bounds__(kPassThreads, 1) k_passes(const __grid_constan
     static_assert(kStage % 128 == 0, "copy alignment");
     const bool computing = threadIdx.x < kTeams * kRun;
     const int team = computing ? (int)threadIdx.x / kRun : ((int)threadIdx.x - kTeams * kRun) / 32;
-    if (team >= kTeams) {            // fills the last warpgroup
-        set_regs<kAuxRegs<T>, false>();
+    // one instruction for all warps of the last warpgroup, also those that only fill it
+    if (!computing) set_regs<kAuxRegs<T>, false>();
+    if (team >= kTeams) {
         __syncthreads();
         return;
     }
@@ -502,7 +503,6 @@ __global__ void __launch_bounds__(kPassThreads, 1) k_passes(const __grid_constan
 
     if (!computing) {
         // ---- scheduling warp
-        set_regs<kAuxRegs<T>, false>();
         __syncthreads();
         // what pass M reads stays in the L2 for pass X, which reads it last
         unsigned long long keep, drop;
@@ -576,9 +576,10 @@ __global__ void __launch_bounds__(kPassThreads, 1) k_passes(const __grid_constan
             if (jobs >= 2 && !expired && !mbar_wait(jfree + 8 * e, ((jobs >> 1) - 1) & 1u)) expired = true;
             s_job[e].pass = kPassEnd;
             mbar_arrive(jfull + 8 * e);
-            // copies may still be in flight where a wait expired: the last one is
-            // waited for, bounded, before the block's shared memory goes
-            if (expired && runs > 0) mbar_wait(full + 8 * ((runs - 1) & 1), ((runs - 1) >> 1) & 1u);
+            // copies may still be in flight where a wait expired: the last one of each
+            // stage is waited for, bounded, before the block's shared memory goes
+            for (u32 q = 1; expired && q <= 2 && q <= runs; ++q)
+                mbar_wait(full + 8 * ((runs - q) & 1), ((runs - q) >> 1) & 1u);
         }
         if (expired) atomicOr(A.status, kFlagTimeout);
         return;
