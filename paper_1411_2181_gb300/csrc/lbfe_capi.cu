@@ -144,7 +144,7 @@ struct lbfe_handle {
     std::vector<int> item_off_h;
     std::vector<lbfe::PopMaps> maps;
     lbfe::StepMaps *maps_dev = nullptr;
-    int total_items = 0, fused_grid = 0, tile_y = 16, z_chunk_req = 0, num_sms = 0, blocks_per_sm = 0;
+    int total_items = 0, fused_grid = 0, tile_y = 16, z_chunk_req = 0, num_sms = 0, blocks_per_sm = 0, device = -1;
     int step_kernel = LBFE_STEP_CELL;
     int advection = 0;               // lbfe_params::advection of every instance
     bool passes_tuned = false;       // ... because lbfe_tune said so
@@ -465,9 +465,8 @@ lbfe_status lbfe_create(lbfe_handle **hp, const lbfe_params *p, int n, void *dev
     if (e == cudaSuccess) e = cudaMemsetAsync(h->status, 0, sizeof(unsigned) * (4 + 3 * (size_t)n), h->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(h->base + L.pass_off[0], 0, L.total - L.pass_off[0], h->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
-    int dev = 0;
-    if (e == cudaSuccess) e = cudaGetDevice(&dev);
-    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&h->num_sms, cudaDevAttrMultiProcessorCount, dev);
+    if (e == cudaSuccess) e = cudaGetDevice(&h->device);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&h->num_sms, cudaDevAttrMultiProcessorCount, h->device);
     if (e != cudaSuccess) {
         delete h;
         return cuda_fail(e, "lbfe_create");
@@ -692,19 +691,42 @@ lbfe_status lbfe_columns_bytes(const lbfe_handle *h, int k, int nx, size_t *byte
     return LBFE_OK;
 }
 
+// Whether [p, p + bytes) lies in one allocation of device dev.
+static bool device_range(const void *p, size_t bytes, int dev) {
+    using range_fn = CUresult (*)(CUdeviceptr *, size_t *, CUdeviceptr);
+    static const range_fn fn = [] {
+        void *f = nullptr;
+        cudaDriverEntryPointQueryResult q = cudaDriverEntryPointSymbolNotFound;
+        if (cudaGetDriverEntryPointByVersion("cuMemGetAddressRange", &f, 12000, cudaEnableDefault, &q) != cudaSuccess)
+            cudaGetLastError();
+        return q == cudaDriverEntryPointSuccess ? (range_fn)f : nullptr;
+    }();
+    cudaPointerAttributes at;
+    if (cudaPointerGetAttributes(&at, p) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    CUdeviceptr start = 0;
+    size_t size = 0;
+    return at.type == cudaMemoryTypeDevice && at.device == dev && fn &&
+           fn(&start, &size, (CUdeviceptr)p) == CUDA_SUCCESS && (CUdeviceptr)p - start <= size &&
+           bytes <= size - ((CUdeviceptr)p - start);
+}
+
 static lbfe_status copy_columns(lbfe_handle *h, int k, int x0, int nx, char *dev, bool get) {
     if (!h || k < 0 || k >= h->n || !dev || nx < 1 || x0 < 0) return LBFE_ERR_BAD_PARAM;
     const InstDev &I = h->inst[k];
     if (x0 + nx > I.Lx) return LBFE_ERR_BAD_PARAM;
     if (!h->ready[k]) return LBFE_ERR_STATE;
-    // a buffer in this device's memory is copied by one kernel; any other the
-    // copy engine can reach (another device's, pinned host memory) array by array
-    cudaPointerAttributes at;
+    // a buffer in one allocation of the handle's device, with that device
+    // current, is copied by one kernel; any other the copy engine can reach
+    // (another device's, pinned host memory) array by array, and what it
+    // refuses stays refused
     int device = -1;
     CK(cudaGetDevice(&device));
-    if (cudaPointerGetAttributes(&at, dev) != cudaSuccess)
-        cudaGetLastError();
-    else if (at.type == cudaMemoryTypeDevice && at.device == device) {
+    const size_t cell = 2 * lbfe::Q * elem_bytes(h->precision) + 6 * sizeof(float) +
+                        (h->precision != LBFE_FP32 && I.dens[0] ? sizeof(float2) : 0);
+    if (device == h->device && device_range(dev, (size_t)nx * I.Ly * I.Lz * cell, device)) {
         CK(lbfe::launch_columns(h->ctx(), k, h->cur, x0, nx, dev, get));
         return LBFE_OK;
     }
