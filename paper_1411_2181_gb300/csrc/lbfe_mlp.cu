@@ -667,14 +667,15 @@ lbfe_status lbfe_mlp_epoch(lbfe_mlp *m, const float *x_dev, const float *t_dev, 
         return LBFE_ERR_BAD_PARAM;
     double *losses = (double *)(m->base + m->L.losses), host[kEpochLosses];
     double total = 0.0;
-    int first = 0, n = 0;            // row of losses[0], batches since
+    long long first = 0;             // row of losses[0]
+    int n = 0;                       // batches since
     auto read = [&]() {
         if (!loss_sum_host || n == 0) return cudaSuccess;
         cudaError_t e = cudaMemcpyAsync(host, losses, sizeof(double) * n, cudaMemcpyDeviceToHost, m->stream);
         if (e == cudaSuccess) e = cudaStreamSynchronize(m->stream);
         if (e != cudaSuccess) return e;
         for (int k = 0; k < n; ++k, first += batch) {
-            const int B = rows - first < batch ? rows - first : batch;
+            const int B = (int)(rows - first < batch ? rows - first : batch);
             total += (double)(float)(host[k] / B) * B;
         }
         n = 0;

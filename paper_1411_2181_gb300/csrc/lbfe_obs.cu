@@ -17,8 +17,8 @@
 //   [6 Lx] sums, mass A, mass B (FP64 bits), status word, finished blocks.
 // Measured on 192 x 96 x 80 in FP32, call to result: 256 us with one block
 // per row of x-planes, shared-memory sums in the loop, a one-thread sum of
-// the masses and three copies; 76 us now, 54 us of it this kernel (4.2 TB/s;
-// floor 33 us).
+// the masses and three copies; 71 to 76 us now, about 50 us of it this kernel
+// (floor 33 us).
 #include "lbfe_internal.cuh"
 
 namespace lbfe {
@@ -128,7 +128,7 @@ cudaError_t launch_observables(const InstDev &I, int precision, int cur, unsigne
     cudaError_t e = cudaMemsetAsync(I.prof, 0, sizeof(unsigned long long) * obs_words(I.Lx), stream);
     if (e != cudaSuccess) return e;
     const int tiles = (I.Lx + 31) / 32;
-    // blocks of eight rows at a time, four blocks on an SM
+    // blocks of eight rows at a time, three blocks on an SM
     const long long rows = (long long)I.Ly * I.Lz;
     const long long most = kObsBlocks / tiles, want = (rows + kObsWarps - 1) / kObsWarps;
     const dim3 grid((unsigned)tiles, (unsigned)(want < most ? want : most));
