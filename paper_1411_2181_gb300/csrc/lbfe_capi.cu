@@ -192,16 +192,27 @@ struct lbfe_handle {
     }
 };
 
-// Depth of the z-chunks: the one with the fewest planes marched by the busiest
+// Depth of the z-chunks: the one with the least estimated time of the busiest
 // block (a chunk costs four planes more than it holds).  Items of one lattice
 // are equal and start together, so that they march in waves of the resident
-// blocks; the items of a batch are handed out as blocks become free, and what
-// that leaves uneven came to about two items (below: 523, 485 and 438 planes'
-// time at 93, 49 and 27 planes a chunk).  Chunks of at least 8 planes.
-// Measured, us per step, chunks that fill the blocks about once -> this:
-// 256 x 128 x 64 FP16 (12 rows; 88 columns) 307 -> 212, twelve uneven lattices
-// FP16 2234 -> 1870; 192 x 96 x 80 keeps its 40 (FP32) and 27 planes (FP16).
-static int auto_z_chunk(const std::vector<InstDev> &inst, long long slots) {
+// blocks, at the same pace.  The items of a batch are handed out as blocks become
+// free, and neighbours that started together drift apart over a deep chunk (tiles
+// at a seam or an edge take another time per plane), until the planes they share
+// are no longer in the L2: the time of a plane grows with the depth of the chunks
+// (drift_planes), and what the end leaves uneven comes to half an item.
+// Chunks of at least 8 planes.  Measured, us per step: 256 x 128 x 64 FP16
+// (12 rows; 88 columns), chunks that fill the blocks about once -> waves 307 -> 212;
+// 192 x 96 x 80 keeps its 40 (FP32) and 27 planes (FP16).  Batches at 8, 12, 16,
+// 27 and 64 planes a chunk: twelve uneven lattices FP16 1885, 1755, 1715, 1870
+// and 2275, FP32 2039, 1960, 2005, 2310 and 2957; 32 of them FP16 4192, 3882,
+// 3845, 4173 and 5003; 40 boxes of 40 planes FP16 2340, 2289, 2226, 2279 and 2170,
+// at 20 planes 2042.
+static double drift_planes(const lbfe_handle *h) { return h->precision == LBFE_FP32 ? 43.0 : 86.0; }
+// A plane of items that all start together takes 3.2 us (FP32, 4.4 with 2-byte
+// storage), one of a batch's about 2.3 (3.2) and what the drift adds.
+constexpr double kTogether = 1.4;
+
+static int auto_z_chunk(const std::vector<InstDev> &inst, long long slots, double drift) {
     int lz = 0, best = 8;
     for (auto &I : inst) lz = std::max(lz, I.Lz);
     double best_cost = 0.0;
@@ -218,7 +229,7 @@ static int auto_z_chunk(const std::vector<InstDev> &inst, long long slots) {
         double cost = deepest;
         if (items > slots)
             cost = inst.size() == 1 ? (double)deepest * ((items + slots - 1) / slots)
-                                    : (double)planes / slots + 2.0 * deepest;
+                                    : ((double)planes / slots + 0.5 * deepest) * (1.0 + (deepest - 4) / drift) / kTogether;
         if (best_cost == 0.0 || cost < best_cost) {
             best_cost = cost;
             best = zc;
@@ -249,7 +260,7 @@ static lbfe_status configure_fused(lbfe_handle *h, int step_kernel, int tile_y, 
         I.nty = (I.Ly + tile_y - 1) / tile_y;
     }
     const long long slots = (long long)h->num_sms * bps;
-    const int zc_auto = z_chunk == 0 ? auto_z_chunk(h->inst, slots) : 0;
+    const int zc_auto = z_chunk == 0 ? auto_z_chunk(h->inst, slots, drift_planes(h)) : 0;
     std::vector<int> off(h->n + 1, 0);
     for (int k = 0; k < h->n; ++k) {
         InstDev &I = h->inst[k];
@@ -299,10 +310,10 @@ static bool passes_possible(const lbfe_handle *h) {
 
 // Whether a new handle's steps run in three passes instead of tiles: the
 // smaller estimate of a step's time (the fields are the same bit for bit).
-//   tiles   planes that the busiest block marches, 3.2 us each (8 rows, FP32;
-//           3.6 in batches), 4.4 (12 rows, 2-byte storage), 3.7 (second-order
-//           advection), half as much again where rows are no 16-byte
-//           multiples (no copies);
+//   tiles   planes that the busiest block marches, 3.2 us each (8 rows, FP32),
+//           4.4 (12 rows, 2-byte storage), 3.7 (second-order advection), in
+//           batches as auto_z_chunk says, half as much again where rows are no
+//           16-byte multiples (no copies);
 //   passes  about 8 us of launch and dependent passes, 0.5 ns a cell of the
 //           largest plane (a pass stays two planes behind the one before) and
 //           0.100 ns a cell (FP32), 0.105 (FP16), 0.112 (BF16), 0.15
@@ -312,24 +323,27 @@ static bool passes_possible(const lbfe_handle *h) {
 // 37 / 32 (FP16 51 / 45), 141 x 75 x 53 103 / 62 (FP16 101 / 75), 40 x 128 x 90
 // 94 / 53, 128 x 128 x 16 37 / 41, 100 x 96 x 80 109 / 83 (FP16 141 / 87), 192 x 96 x 80 142 / 160
 // (FP16 140 / 165, BF16 145 / 175, second order 160 / 233), 256 x 128 x 64
-// 212 / 235, sixteen 320 x 44 x 40 1024 / 972 (FP16 853 / 1076),
-// twelve uneven lattices 2345 / 1987 (FP16 1874 / 2074).
+// 212 / 235, sixteen 320 x 44 x 40 995 / 973 (FP16 850 / 1079), forty 2444 / 2430,
+// twelve uneven lattices 1961 / 1986 (FP16 1714 / 2078, second order 2079 / 2823),
+// four of them 686 / 636, 32 of them 4297 / 4390.
 static bool prefer_passes(const lbfe_handle *h) {
     const bool fp32 = h->precision == LBFE_FP32;
-    double planes = 0.0, most = 0.0, cells = 0.0, plane = 0.0;
+    double planes = 0.0, most = 0.0, cells = 0.0, plane = 0.0, depth = 0.0;
     for (int k = 0; k < h->n; ++k) {
         const InstDev &I = h->inst[k];
         const double w = h->maps[k].ok ? 1.0 : 1.5;
         planes += w * I.ntx * I.nty * (I.Lz + 4.0 * I.nzc);
         most = std::max(most, w * (I.zc + 4.0));
+        depth = std::max(depth, (double)I.zc);
         cells += (double)I.N;
         plane = std::max(plane, (double)I.Lx * I.Ly);
     }
     const double slots = (double)h->num_sms * h->blocks_per_sm;
     double march = most;
     if (h->total_items > slots)
-        march = h->n == 1 ? most * std::ceil(h->total_items / slots) : planes / slots + most;
-    const double tile = march * (h->advection ? 3.7 : (fp32 ? (h->n > 1 ? 3.6 : 3.2) : 4.4));
+        march = h->n == 1 ? most * std::ceil(h->total_items / slots)
+                          : (planes / slots + 0.5 * most) * (1.0 + depth / drift_planes(h)) / kTogether;
+    const double tile = march * (h->advection ? 3.7 : (fp32 ? 3.2 : 4.4));
     const double ns = h->advection ? 0.15 : (fp32 ? 0.100 : (h->precision == LBFE_FP16_OFFSET ? 0.105 : 0.112));
     return 8.0 + 0.5e-3 * plane + 1e-3 * ns * (h->n > 1 ? 1.1 : 1.0) * cells < tile;
 }
