@@ -229,14 +229,16 @@ def measured_peak():
 
 # sources of the step kernels (device code and their launch code); a
 # profile summary stays valid while these are unchanged
-STEP_SOURCES = ("lbfe_internal.cuh", "lbfe_step.cuh", "lbfe_fused.cu", "lbfe_fused2.cu", "lbfe_passes.cu")
+STEP_SOURCES = ("lbfe_internal.cuh", "lbfe_step.cuh", "lbfe_fused.cu", "lbfe_fused2.cu")
+PASSES_SOURCES = ("lbfe_internal.cuh", "lbfe_step.cuh", "lbfe_passes.cu")
 
 
-def kernel_source_hash():
-    """Hash of the step-kernel sources with comments and layout removed, so
-    that a profile summary survives edits to comments only."""
+def kernel_source_hash(kernel: int = 0):
+    """Hash of the sources of the tile kernels or (kernel 2) the three-pass
+    kernel with comments and layout removed, so that a profile summary
+    survives edits to comments only."""
     h = hashlib.sha256()
-    for fn in STEP_SOURCES:
+    for fn in PASSES_SOURCES if kernel == 2 else STEP_SOURCES:
         src = open(os.path.join(ROOT, "paper_1411_2181_gb300", "csrc", fn)).read()
         src = re.sub(r"/\*.*?\*/", "", src, flags=re.S)
         src = re.sub(r"//[^\n]*", "", src)
@@ -256,7 +258,7 @@ def profiled_traffic(workload_name: str, precision: int, advection: int = 0, ker
     txt = open(fn).read()
     m_h = re.search(r"kernel source hash:\s*`?([0-9a-f]{16})", txt)
     m_b = re.search(r"dram bytes per lattice update:\s*([0-9.]+)", txt)
-    if not m_h or not m_b or m_h.group(1) != kernel_source_hash():
+    if not m_h or not m_b or m_h.group(1) != kernel_source_hash(kernel):
         return None, fn
     return float(m_b.group(1)), fn
 
