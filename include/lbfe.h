@@ -274,8 +274,8 @@ lbfe_status lbfe_launch_config(const lbfe_handle *h, int *step_kernel, int *tile
 #define LBFE_INJECT_SHORT_COPIES 1u
 /* what = LBFE_INJECT_LOST_COUNTS: with LBFE_STEP_PASSES the first pass of a
  * step is not counted as finished, so that the second pass's bounded waits for
- * it expire (about one second); every team then runs through its slots without
- * waiting and lbfe_check reports LBFE_ERR_TIMEOUT.  SHORT_COPIES makes the
+ * it expire (about one second); every team then takes no further slot, the
+ * launch ends and lbfe_check reports LBFE_ERR_TIMEOUT.  SHORT_COPIES makes the
  * handle step with the tile kernels. */
 #define LBFE_INJECT_LOST_COUNTS 2u
 lbfe_status lbfe_test_inject(lbfe_handle *h, unsigned what);

@@ -513,6 +513,11 @@ __global__ void __launch_bounds__(kPassThreads, 1) k_passes(const __grid_constan
             if (t == 0) next = (int)atomicAdd(A.work, 1u);
             return __shfl_sync(0xffffffffu, next, 0);
         };
+        // the place of the next job, once its last one has been read
+        auto job_slot = [&]() { return jobs < 2 || mbar_wait(jfree + 8 * (jobs & 1), ((jobs >> 1) - 1) & 1u); };
+        // The warp stops at its first expired wait: a job or a copy handed over
+        // without that wait would overwrite one that is still being read.  runs and
+        // jobs (lane 0) are what was handed over.
         for (int slot = take(); slot < A.slots; slot = take()) {
             const int pass = slot % 3;
             const int q = slot / 3 - (pass == 0 ? 0 : (pass == 1 ? A.lag_x : A.lag_u));
@@ -542,21 +547,26 @@ __global__ void __launch_bounds__(kPassThreads, 1) k_passes(const __grid_constan
                         if (!ok) expired = true;
                     }
                     __threadfence();
-                    __syncwarp();
+                    if (__any_sync(0xffffffffu, expired)) {
+                        expired = true;
+                        break;
+                    }
                 }
-                if (t == 0) {
+                if (t == 0 && !job_slot()) expired = true;
+                if (t == 0 && !expired) {
                     const int e = jobs & 1;
-                    if (jobs >= 2 && !expired && !mbar_wait(jfree + 8 * e, ((jobs >> 1) - 1) & 1u)) expired = true;
                     s_job[e] = Job{pass, k, step, c0, c1};
                     mbar_arrive(jfull + 8 * e);
+                    ++jobs;
                     if (pass < 2) {
                         const CUtensorMap *map = I.runs[(A.parity + step) & 1];
                         asm volatile("fence.proxy.async;" ::: "memory");
-                        for (u32 c = c0; c < c1; c += kRun, ++runs) {
+                        for (u32 c = c0; c < c1; c += kRun) {
                             const int sg = runs & 1;
-                            if (runs >= 2 && !expired && !mbar_wait(freeb + 8 * sg, ((runs >> 1) - 1) & 1u))
+                            if (runs >= 2 && !mbar_wait(freeb + 8 * sg, ((runs >> 1) - 1) & 1u)) {
                                 expired = true;
-                            if (expired) continue;
+                                break;
+                            }
                             asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
                             mbar_expect(full + 8 * sg, kStage);
                             asm volatile(
@@ -565,21 +575,25 @@ __global__ void __launch_bounds__(kPassThreads, 1) k_passes(const __grid_constan
                                 "l"(reinterpret_cast<unsigned long long>(map)), "r"((int)c), "r"(0),
                                 "r"(full + 8 * sg), "l"(pass == 0 ? keep : drop)
                                 : "memory");
+                            ++runs;
                         }
                     }
                 }
-                ++jobs;
+                if (__any_sync(0xffffffffu, expired)) break;
             }
         }
         if (t == 0) {
-            const int e = jobs & 1;
-            if (jobs >= 2 && !expired && !mbar_wait(jfree + 8 * e, ((jobs >> 1) - 1) & 1u)) expired = true;
-            s_job[e].pass = kPassEnd;
-            mbar_arrive(jfull + 8 * e);
-            // copies may still be in flight where a wait expired: the last one of each
-            // stage is waited for, bounded, before the block's shared memory goes
-            for (u32 q = 1; expired && q <= 2 && q <= runs; ++q)
-                mbar_wait(full + 8 * ((runs - q) & 1), ((runs - q) >> 1) & 1u);
+            if (job_slot()) {
+                s_job[jobs & 1].pass = kPassEnd;
+                mbar_arrive(jfull + 8 * (jobs & 1));
+            } else {
+                expired = true;      // the team's own wait for its next job ends it
+            }
+            // copies may still be in flight where a wait expired, here or in the computing
+            // warps: the last one issued to each stage is waited for, bounded, before the
+            // block's shared memory goes (at once where the computing warps have seen it)
+            for (u32 q = 1; q <= 2 && q <= runs; ++q)
+                if (!mbar_wait(full + 8 * ((runs - q) & 1), ((runs - q) >> 1) & 1u)) expired = true;
         }
         if (expired) atomicOr(A.status, kFlagTimeout);
         return;
@@ -596,10 +610,13 @@ __global__ void __launch_bounds__(kPassThreads, 1) k_passes(const __grid_constan
             const int e = jobs & 1;
             bool known = false;
             for (int tries = 0; tries < 4 && !known; ++tries) known = mbar_wait(jfull + 8 * e, (jobs >> 1) & 1u);
-            if (!known) expired = true;
-            t_cur[team] = s_job[e];
-            if (!known) t_cur[team].pass = kPassEnd;
-            mbar_arrive(jfree + 8 * e);
+            if (known) {
+                t_cur[team] = s_job[e];
+                mbar_arrive(jfree + 8 * e);
+            } else {
+                t_cur[team].pass = kPassEnd;
+                expired = true;
+            }
         }
         team_barrier();
         const Job J = t_cur[team];
@@ -623,7 +640,9 @@ __global__ void __launch_bounds__(kPassThreads, 1) k_passes(const __grid_constan
                 else
                     pass_x<T>(I, b, min(n, c1 - 1), n < c1, seed, A.status, st, wait);
                 __syncwarp();
-                if ((t & 31) == 0) mbar_arrive(freeb + 8 * sg);
+                // a stage whose copy was not seen to arrive is never handed back: the
+                // scheduling warp's wait for it expires and it copies no more
+                if ((t & 31) == 0 && !expired) mbar_arrive(freeb + 8 * sg);
             }
         } else {
             for (u32 c = c0; c < c1; c += kRun) pass_u<ADV2>(I, b, min(c + t, c1 - 1), c + t < c1, A.status);

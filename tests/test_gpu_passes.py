@@ -190,3 +190,30 @@ def test_two_handles_on_two_streams(L):
         for s in hs:
             s.close()
     assert all(np.array_equal(a, b) for a, b in zip(*out))
+
+
+@pytest.mark.parametrize("prec", [0, 1])
+@pytest.mark.parametrize("shapes", [[(141, 75, 9)], [(256, 128, 12)], [(7, 5, 6), (256, 128, 12), (33, 17, 11)]])
+def test_a_launch_stops_at_expired_waits(L, shapes, prec):
+    """Waits expire with jobs handed over and copies of both stages issued
+    (slots of one and of four runs, one and several steps, small and large
+    lattices in a batch): the launch ends with a status, no job or copy is
+    overwritten, and the blocks that take the shared memory over next, at
+    once on the same stream, compute the right fields."""
+    import time
+    ps = [params(L, sh, prec, 0, 1) for sh in shapes]
+    st = [random_populations(sh, seed=3, amp=0.01) for sh in shapes]
+    ref = solver(L, ps, (8, 0, 0), st)
+    ref.step(3)
+    for steps in (1, 2, 5):
+        s, nxt = (solver(L, ps, (8, 0, L.STEP_PASSES), st) for _ in range(2))
+        s.test_inject(L.INJECT_LOST_COUNTS)
+        t0 = time.time()
+        s.step(steps)
+        nxt.step(3)
+        assert s.check() == L.ERR_TIMEOUT and time.time() - t0 < 30.0
+        assert nxt.check() == L.OK
+        same(L, nxt, ref, len(shapes))
+        s.close()
+        nxt.close()
+    ref.close()
