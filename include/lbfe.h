@@ -275,8 +275,9 @@ lbfe_status lbfe_launch_config(const lbfe_handle *h, int *step_kernel, int *tile
 /* what = LBFE_INJECT_LOST_COUNTS: with LBFE_STEP_PASSES the first pass of a
  * step is not counted as finished, so that the second pass's bounded waits for
  * it expire (about one second); every team then takes no further slot, the
- * launch ends and lbfe_check reports LBFE_ERR_TIMEOUT.  SHORT_COPIES makes the
- * handle step with the tile kernels. */
+ * launch ends and lbfe_check reports LBFE_ERR_TIMEOUT (for the rest of the
+ * handle's life).  what = 0 undoes it: initialised again, the handle steps as
+ * before.  SHORT_COPIES makes the handle step with the tile kernels. */
 #define LBFE_INJECT_LOST_COUNTS 2u
 lbfe_status lbfe_test_inject(lbfe_handle *h, unsigned what);
 

@@ -82,11 +82,13 @@ struct PassArgs {
     int period, lag_x, lag_u;        // distance of two steps; of the passes of a step
     int slots;
     int lost;                        // test hook: pass M is not counted
-    unsigned *status, *work;
+    unsigned *status;
+    unsigned *work;                  // [0] slots taken, [1] finished teams, kGaveUp; zero between launches
     int item_off[kStepMaxInst + 1];  // first slot of each instance
     PassInst inst[kStepMaxInst];
 };
 static_assert(sizeof(PassArgs) < 32000, "kernel parameter space");
+constexpr unsigned kGaveUp = 1u << 31;   // a wait of the launch has expired
 
 // n / d by the reciprocal of fast_div.
 __device__ __forceinline__ u32 div_by(u32 n, u32 mul, u32 sh) {
@@ -100,14 +102,20 @@ __device__ __forceinline__ unsigned ld_relaxed(const unsigned *p) {
     return v;
 }
 
-// Wait until *p has reached target; false once the wait expired (here, or
-// anywhere: the launch's status word tells).
-__device__ __forceinline__ bool wait_count(const unsigned *p, unsigned target, unsigned *status) {
+// Report an expired wait to the host and to the launch's other waits.
+__device__ __forceinline__ void give_up(const PassArgs &A) {
+    atomicOr(A.status, kFlagTimeout);
+    atomicOr(A.work + 1, kGaveUp);
+}
+
+// Wait until *p has reached target; false once a wait of the launch expired,
+// here or anywhere.
+__device__ __forceinline__ bool wait_count(const unsigned *p, unsigned target, const PassArgs &A) {
     unsigned long long t0 = 0;
     for (u32 it = 0; it < kWaitRounds; ++it) {
         if ((int)(ld_relaxed(p) - target) >= 0) return true;
         if ((it & 255u) == 255u) {
-            if (ld_relaxed(status) & kFlagTimeout) return false;
+            if (ld_relaxed(A.work + 1) & kGaveUp) return false;
             const unsigned long long now = global_ns();
             if (t0 == 0)
                 t0 = now;
@@ -115,7 +123,7 @@ __device__ __forceinline__ bool wait_count(const unsigned *p, unsigned target, u
                 break;
         }
     }
-    atomicOr(status, kFlagTimeout);
+    give_up(A);
     return false;
 }
 
@@ -471,7 +479,7 @@ __global__ void __launch_bounds__(kPassThreads, 1) k_passes(const __grid_constan
     // per team, two of each: run copied, run read, job known, job read
     __shared__ __align__(8) unsigned long long t_full[kTeams][2], t_free[kTeams][2], t_jfull[kTeams][2],
         t_jfree[kTeams][2];
-    __shared__ bool t_last[kTeams];
+    __shared__ int t_how[kTeams];
     constexpr u32 kStage = (u32)(2 * Q * kRun * sizeof(T));
     static_assert(kStage % 128 == 0, "copy alignment");
     const bool computing = threadIdx.x < kTeams * kRun;
@@ -497,7 +505,6 @@ __global__ void __launch_bounds__(kPassThreads, 1) k_passes(const __grid_constan
         }
     }
     const u32 cells = (u32)(kRun * A.R);
-    const int workers = (int)gridDim.x * kTeams;
     bool expired = false;
     u32 runs = 0, jobs = 0;          // runs staged, jobs taken so far
 
@@ -509,8 +516,8 @@ __global__ void __launch_bounds__(kPassThreads, 1) k_passes(const __grid_constan
         asm volatile("createpolicy.fractional.L2::evict_last.b64 %0, 1.0;" : "=l"(keep));
         asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(drop));
         auto take = [&]() {
-            int next = 0;
-            if (t == 0) next = (int)atomicAdd(A.work, 1u);
+            int next = A.slots;
+            if (t == 0 && !expired) next = (int)atomicAdd(A.work, 1u);
             return __shfl_sync(0xffffffffu, next, 0);
         };
         // the place of the next job, once its last one has been read
@@ -541,18 +548,15 @@ __global__ void __launch_bounds__(kPassThreads, 1) k_passes(const __grid_constan
                     const unsigned prev = ld_relaxed(I.cnt + 3 * Lz) + (unsigned)step * I.LxLy, now = prev + I.LxLy;
                     for (int z = zl + t; z <= zh && !expired; z += 32) {
                         bool ok = true;
-                        if (pass == 1) ok = wait_count(I.cnt + z, now, A.status);
-                        if (pass == 2 || (pass == 0 && ok)) ok = wait_count(I.cnt + Lz + z, pass == 2 ? now : prev, A.status);
-                        if (pass < 2 && ok && step > 0) ok = wait_count(I.cnt + 2 * Lz + z, prev, A.status);
+                        if (pass == 1) ok = wait_count(I.cnt + z, now, A);
+                        if (pass == 2 || (pass == 0 && ok)) ok = wait_count(I.cnt + Lz + z, pass == 2 ? now : prev, A);
+                        if (pass < 2 && ok && step > 0) ok = wait_count(I.cnt + 2 * Lz + z, prev, A);
                         if (!ok) expired = true;
                     }
                     __threadfence();
-                    if (__any_sync(0xffffffffu, expired)) {
-                        expired = true;
-                        break;
-                    }
+                    expired = __any_sync(0xffffffffu, expired);
                 }
-                if (t == 0 && !job_slot()) expired = true;
+                if (t == 0 && !expired && !job_slot()) expired = true;
                 if (t == 0 && !expired) {
                     const int e = jobs & 1;
                     s_job[e] = Job{pass, k, step, c0, c1};
@@ -579,23 +583,21 @@ __global__ void __launch_bounds__(kPassThreads, 1) k_passes(const __grid_constan
                         }
                     }
                 }
-                if (__any_sync(0xffffffffu, expired)) break;
             }
         }
         if (t == 0) {
-            if (job_slot()) {
-                s_job[jobs & 1].pass = kPassEnd;
-                mbar_arrive(jfull + 8 * (jobs & 1));
-            } else {
-                expired = true;      // the team's own wait for its next job ends it
-            }
             // copies may still be in flight where a wait expired, here or in the computing
             // warps: the last one issued to each stage is waited for, bounded, before the
             // block's shared memory goes (at once where the computing warps have seen it)
             for (u32 q = 1; q <= 2 && q <= runs; ++q)
                 if (!mbar_wait(full + 8 * ((runs - q) & 1), ((runs - q) >> 1) & 1u)) expired = true;
+            if (expired) give_up(A);
+            // the end is the last that the team hears of this warp
+            if (job_slot()) {
+                s_job[jobs & 1].pass = kPassEnd;
+                mbar_arrive(jfull + 8 * (jobs & 1));
+            }
         }
-        if (expired) atomicOr(A.status, kFlagTimeout);
         return;
     }
 
@@ -605,11 +607,12 @@ __global__ void __launch_bounds__(kPassThreads, 1) k_passes(const __grid_constan
     auto team_barrier = [&]() { asm volatile("bar.sync %0, 256;" ::"r"(1 + team) : "memory"); };
     for (;; ++jobs) {
         // one thread takes the job, so that the team agrees on it (and on its end)
-        // whatever the waits do; the scheduling warp's own waits come first
+        // whatever the waits do; the scheduling warp's own waits come first, and have
+        // all ended, with the warp, before this one expires
         if (t == 0) {
             const int e = jobs & 1;
             bool known = false;
-            for (int tries = 0; tries < 4 && !known; ++tries) known = mbar_wait(jfull + 8 * e, (jobs >> 1) & 1u);
+            for (int tries = 0; tries < 16 && !known; ++tries) known = mbar_wait(jfull + 8 * e, (jobs >> 1) & 1u);
             if (known) {
                 t_cur[team] = s_job[e];
                 mbar_arrive(jfree + 8 * e);
@@ -660,19 +663,26 @@ __global__ void __launch_bounds__(kPassThreads, 1) k_passes(const __grid_constan
             }
         }
     }
-    if (expired) atomicOr(A.status, kFlagTimeout);
+    if (expired) give_up(A);
     // the last team leaves the counters as the next launch expects them
     team_barrier();
     if (t == 0) {
         __threadfence();
-        t_last[team] = atomicAdd(A.work + 1, 1u) == (unsigned)workers - 1;
+        const unsigned n = atomicAdd(A.work + 1, 1u);
         __threadfence();
+        // 1, or 2 if the launch gave up
+        t_how[team] = (n & ~kGaveUp) != (unsigned)kTeams * gridDim.x - 1u ? 0 : (n & kGaveUp ? 2 : 1);
     }
     team_barrier();
-    if (!t_last[team]) return;
+    const int how = t_how[team];
+    if (how == 0) return;
     for (int k = t; k < A.n; k += kRun) {
         const PassInst &I = A.inst[k];
-        I.cnt[3 * I.Lz] += (unsigned)A.steps * I.LxLy;
+        const u32 base = I.cnt[3 * I.Lz] + (unsigned)A.steps * I.LxLy;
+        // a launch that gave up has left slots uncounted: the counts are set to what they
+        // would have reached, so that the next launch waits for its own slots alone
+        for (int z = 0; how == 2 && z < 3 * I.Lz; ++z) I.cnt[z] = base;
+        I.cnt[3 * I.Lz] = base;
         if (I.step_ctr) I.step_ctr[(A.parity + A.steps) & 1] = __ldcg(I.step_ctr + A.parity) + (unsigned)A.steps;
     }
     if (t == 0) {

@@ -217,3 +217,36 @@ def test_a_launch_stops_at_expired_waits(L, shapes, prec):
         s.close()
         nxt.close()
     ref.close()
+
+
+@pytest.mark.parametrize("prec", [0, 2])
+def test_a_handle_steps_again_after_expired_waits(L, prec):
+    """A launch that gave up leaves its counters as if every slot had been
+    counted: the same handle, its hook undone and initialised again, steps in
+    order, at once, with the tile kernel's bits (70 instances: two launches a
+    step).  The status keeps telling of the expired wait."""
+    import time
+    rng = np.random.default_rng(11)
+    shapes = [(141, 75, 9), (256, 64, 12)] + [(int(rng.integers(1, 40)), int(rng.integers(1, 30)), int(rng.integers(2, 20)))
+                                              for _ in range(68)]
+    ps = [params(L, sh, prec, 0, k % 3) for k, sh in enumerate(shapes)]
+    st = [random_populations(sh, seed=k, amp=0.01) for k, sh in enumerate(shapes)]
+    s, ref = solver(L, ps, (8, 0, L.STEP_PASSES), st), solver(L, ps, (8, 0, 0), st)
+    for lost in (1, 3):
+        s.test_inject(L.INJECT_LOST_COUNTS)
+        s.step(lost)
+        assert s.check() == L.ERR_TIMEOUT
+        s.test_inject(0)
+        for h in (s, ref):
+            for k, (p, (f, C)) in enumerate(zip(ps, st)):
+                h.init(k, np.ones((2, p.Lz, p.Ly, p.Lx)))
+                h.set_field(k, L.FIELD_F, f)
+                h.set_field(k, L.FIELD_C, C)
+        t0 = time.time()
+        for n in (1, 4, 18):
+            s.step(n)
+            ref.step(n)
+        assert s.check() == L.ERR_TIMEOUT and time.time() - t0 < 0.5
+        same(L, s, ref, len(shapes))
+    s.close()
+    ref.close()
