@@ -53,7 +53,8 @@ lbfe_status lbfe_mlp_create(lbfe_mlp **m, int max_batch, int weights_bf16, void 
 lbfe_status lbfe_mlp_set_params(lbfe_mlp *m, const float *host_params);
 lbfe_status lbfe_mlp_get_params(lbfe_mlp *m, float *host_params);
 
-/* y[batch][4] = network(x[batch][6]); x and y are device pointers. */
+/* y[batch][4] = network(x[batch][6]); x and y are device pointers and may
+ * overlap.  LBFE_ERR_CUDA if y is known not to hold the result. */
 lbfe_status lbfe_mlp_forward(lbfe_mlp *m, const float *x_dev, int batch, float *y_dev);
 
 /* Loss of a batch and its gradient with respect to the parameters (kept in

@@ -348,6 +348,29 @@ static bool prefer_passes(const lbfe_handle *h) {
     return 8.0 + 0.5e-3 * plane + 1e-3 * ns * (h->n > 1 ? 1.1 : 1.0) * cells < tile;
 }
 
+namespace lbfe {
+bool device_range(const void *p, size_t bytes, int dev) {
+    using range_fn = CUresult (*)(CUdeviceptr *, size_t *, CUdeviceptr);
+    static const range_fn fn = [] {
+        void *f = nullptr;
+        cudaDriverEntryPointQueryResult q = cudaDriverEntryPointSymbolNotFound;
+        if (cudaGetDriverEntryPointByVersion("cuMemGetAddressRange", &f, 12000, cudaEnableDefault, &q) != cudaSuccess)
+            cudaGetLastError();
+        return q == cudaDriverEntryPointSuccess ? (range_fn)f : nullptr;
+    }();
+    cudaPointerAttributes at;
+    if (cudaPointerGetAttributes(&at, p) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    CUdeviceptr start = 0;
+    size_t size = 0;
+    return at.type == cudaMemoryTypeDevice && at.device == dev && fn &&
+           fn(&start, &size, (CUdeviceptr)p) == CUDA_SUCCESS && (CUdeviceptr)p - start <= size &&
+           bytes <= size - ((CUdeviceptr)p - start);
+}
+}  // namespace lbfe
+
 extern "C" {
 
 const char *lbfe_status_str(lbfe_status s) {
@@ -705,28 +728,6 @@ lbfe_status lbfe_columns_bytes(const lbfe_handle *h, int k, int nx, size_t *byte
     return LBFE_OK;
 }
 
-// Whether [p, p + bytes) lies in one allocation of device dev.
-static bool device_range(const void *p, size_t bytes, int dev) {
-    using range_fn = CUresult (*)(CUdeviceptr *, size_t *, CUdeviceptr);
-    static const range_fn fn = [] {
-        void *f = nullptr;
-        cudaDriverEntryPointQueryResult q = cudaDriverEntryPointSymbolNotFound;
-        if (cudaGetDriverEntryPointByVersion("cuMemGetAddressRange", &f, 12000, cudaEnableDefault, &q) != cudaSuccess)
-            cudaGetLastError();
-        return q == cudaDriverEntryPointSuccess ? (range_fn)f : nullptr;
-    }();
-    cudaPointerAttributes at;
-    if (cudaPointerGetAttributes(&at, p) != cudaSuccess) {
-        cudaGetLastError();
-        return false;
-    }
-    CUdeviceptr start = 0;
-    size_t size = 0;
-    return at.type == cudaMemoryTypeDevice && at.device == dev && fn &&
-           fn(&start, &size, (CUdeviceptr)p) == CUDA_SUCCESS && (CUdeviceptr)p - start <= size &&
-           bytes <= size - ((CUdeviceptr)p - start);
-}
-
 static lbfe_status copy_columns(lbfe_handle *h, int k, int x0, int nx, char *dev, bool get) {
     if (!h || k < 0 || k >= h->n || !dev || nx < 1 || x0 < 0) return LBFE_ERR_BAD_PARAM;
     const InstDev &I = h->inst[k];
@@ -740,7 +741,7 @@ static lbfe_status copy_columns(lbfe_handle *h, int k, int x0, int nx, char *dev
     CK(cudaGetDevice(&device));
     const size_t cell = 2 * lbfe::Q * elem_bytes(h->precision) + 6 * sizeof(float) +
                         (h->precision != LBFE_FP32 && I.dens[0] ? sizeof(float2) : 0);
-    if (device == h->device && device_range(dev, (size_t)nx * I.Ly * I.Lz * cell, device)) {
+    if (device == h->device && lbfe::device_range(dev, (size_t)nx * I.Ly * I.Lz * cell, device)) {
         CK(lbfe::launch_columns(h->ctx(), k, h->cur, x0, nx, dev, get));
         return LBFE_OK;
     }

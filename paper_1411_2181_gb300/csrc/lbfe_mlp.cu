@@ -463,7 +463,7 @@ MlpLayout mlp_plan(int B) {
 }  // namespace
 
 struct lbfe_mlp {
-    int max_batch = 0, use16 = 1, steps = 0;
+    int max_batch = 0, use16 = 1, steps = 0, device = -1;
     cudaStream_t stream = nullptr;
     char *base = nullptr;
     MlpLayout L;
@@ -593,7 +593,8 @@ lbfe_status lbfe_mlp_create(lbfe_mlp **mp, int max_batch, int weights_bf16, void
     m->stream = (cudaStream_t)stream;
     m->base = (char *)device_block;
     m->L = mlp_plan(max_batch);
-    cudaError_t e = cudaMemsetAsync(m->base, 0, m->L.A[0], m->stream);
+    cudaError_t e = cudaGetDevice(&m->device);
+    if (e == cudaSuccess) e = cudaMemsetAsync(m->base, 0, m->L.A[0], m->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(m->stream);
     if (e != cudaSuccess) {
         delete m;
@@ -626,7 +627,18 @@ lbfe_status lbfe_mlp_get_params(lbfe_mlp *m, float *host_params) {
 
 lbfe_status lbfe_mlp_forward(lbfe_mlp *m, const float *x_dev, int batch, float *y_dev) {
     if (!m || !x_dev || !y_dev || batch < 1 || batch > m->max_batch) return LBFE_ERR_BAD_PARAM;
-    const cudaError_t e = net<false>(m, x_dev, nullptr, nullptr, batch, y_dev);
+    // The blocks write their rows of y while others still read x.  Where y overlaps x, or
+    // does not lie in one allocation of the network's device, the result goes through the
+    // workspace (the loss gradient's dY) and a copy, which refuses what is no such buffer.
+    const size_t bytes = sizeof(float) * 4 * (size_t)batch;
+    const uintptr_t x0 = (uintptr_t)x_dev, y0 = (uintptr_t)y_dev;
+    const bool apart = y0 + bytes <= x0 || x0 + sizeof(float) * 6 * (size_t)batch <= y0;
+    int device = -1;
+    if (cudaGetDevice(&device) != cudaSuccess) return LBFE_ERR_CUDA;
+    const bool direct = apart && device == m->device && lbfe::device_range(y_dev, bytes, device);
+    float *y = direct ? y_dev : m->f(m->L.dY);
+    cudaError_t e = net<false>(m, x_dev, nullptr, nullptr, batch, y);
+    if (e == cudaSuccess && !direct) e = cudaMemcpyAsync(y_dev, y, bytes, cudaMemcpyDeviceToDevice, m->stream);
     return e == cudaSuccess ? LBFE_OK : LBFE_ERR_CUDA;
 }
 

@@ -150,3 +150,39 @@ def test_epoch_equals_single_steps(M, n, bs, bf16):
         assert np.array_equal(a.get_params(), b.get_params()) and np.array_equal(a.grads(), b.grads())
     assert M._lib.lbfe_mlp_epoch(a._h, *[ct.c_void_p(v.data_ptr()) for v in d], n, bs + 1, 1e-3, 0.9, 0.999, 1e-8, 0.0,
                                  None) != 0
+
+
+@pytest.mark.parametrize("B", [1, 37, 4096])
+@pytest.mark.parametrize("off", [0, 4, 6, 20])
+def test_outputs_over_the_inputs(M, B, off):
+    """y may overlap x: the result is the one of separate buffers, wherever in
+    x's rows it starts."""
+    import ctypes as ct
+    import torch
+    net = M.MLP(max_batch=B)
+    net.set_params(M.init_params(5))
+    x = batch(B, 9)[0]
+    buf = torch.zeros(6 * B + 4 * B + 32, device="cuda")
+    want = torch.zeros(4 * B, device="cuda")
+    for _ in range(3):
+        buf[:6 * B] = torch.from_numpy(x.ravel())
+        torch.cuda.synchronize()
+        assert M._lib.lbfe_mlp_forward(net._h, ct.c_void_p(buf.data_ptr()), B, ct.c_void_p(want.data_ptr())) == 0
+        assert M._lib.lbfe_mlp_forward(net._h, ct.c_void_p(buf.data_ptr()), B, ct.c_void_p(buf.data_ptr() + 4 * off)) == 0
+        torch.cuda.synchronize()
+        assert torch.equal(buf[off:off + 4 * B], want) and want.abs().max() > 0
+
+
+def test_outputs_in_pinned_host_memory(M):
+    """A buffer outside the device takes the copy's path: same bits."""
+    import ctypes as ct
+    import torch
+    net = M.MLP(max_batch=341)
+    net.set_params(M.init_params(5))
+    x = torch.from_numpy(batch(341, 9)[0]).cuda()
+    host, dev = torch.zeros(341, 4).pin_memory(), torch.zeros(341, 4, device="cuda")
+    torch.cuda.synchronize()
+    for y in (host, dev):
+        assert M._lib.lbfe_mlp_forward(net._h, ct.c_void_p(x.data_ptr()), 341, ct.c_void_p(y.data_ptr())) == 0
+    torch.cuda.synchronize()
+    assert torch.equal(dev.cpu(), host)
