@@ -186,3 +186,23 @@ def test_outputs_in_pinned_host_memory(M):
         assert M._lib.lbfe_mlp_forward(net._h, ct.c_void_p(x.data_ptr()), 341, ct.c_void_p(y.data_ptr())) == 0
     torch.cuda.synchronize()
     assert torch.equal(dev.cpu(), host)
+
+
+@pytest.mark.parametrize("B", [4560, 4561, 4577, 8193])
+def test_large_batches_of_fp32_weights(M, B):
+    """At and beyond the batch where FP32 weights go layer by layer, also with
+    the outputs over the inputs: against the reference."""
+    import ctypes as ct
+    import torch
+    net = M.MLP(max_batch=B, bf16=False)
+    p = M.init_params(3)
+    net.set_params(p)
+    x = batch(B, 4)[0]
+    want = R.forward(p.astype(np.float64), x.astype(np.float64))
+    y = net.forward(x)
+    assert np.abs(y - want).max() / np.abs(want).max() < TOL_CHAIN
+    buf = torch.from_numpy(x.ravel()).cuda()
+    torch.cuda.synchronize()
+    assert M._lib.lbfe_mlp_forward(net._h, ct.c_void_p(buf.data_ptr()), B, ct.c_void_p(buf.data_ptr())) == 0
+    torch.cuda.synchronize()
+    assert np.array_equal(buf[:4 * B].cpu().numpy().reshape(B, 4), y)
