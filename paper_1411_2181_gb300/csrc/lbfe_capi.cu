@@ -739,9 +739,14 @@ static lbfe_status copy_columns(lbfe_handle *h, int k, int x0, int nx, char *dev
     // refuses stays refused
     int device = -1;
     CK(cudaGetDevice(&device));
-    const size_t cell = 2 * lbfe::Q * elem_bytes(h->precision) + 6 * sizeof(float) +
-                        (h->precision != LBFE_FP32 && I.dens[0] ? sizeof(float2) : 0);
-    if (device == h->device && lbfe::device_range(dev, (size_t)nx * I.Ly * I.Lz * cell, device)) {
+    const size_t bytes = column_bytes(h, I, nx);
+    // A block at an odd address is copied byte by byte, at 0.5 TB/s (whole rows 0.8); the
+    // copy engine takes 271 us for its 44 copies and then runs at 0.7, so that it is the
+    // faster one for large blocks.  Measured, us, kernel / copies: 191 of 192 columns of
+    // 192 x 96 x 80 FP32 (258 MB) 490 / 361, whole 255 x 127 x 95 (541 MB) 656 / 631, whole
+    // 192 x 96 x 80 319 / 361, two columns 11 / 271.
+    const size_t most = ((uintptr_t)dev & 1) == 0 ? ~(size_t)0 : (nx == I.Lx ? 400u : 128u) * (size_t)1000000;
+    if (bytes <= most && device == h->device && lbfe::device_range(dev, bytes, device)) {
         CK(lbfe::launch_columns(h->ctx(), k, h->cur, x0, nx, dev, get));
         return LBFE_OK;
     }

@@ -130,3 +130,31 @@ def test_column_blocks_through_pinned_host_memory(L):
     torch.cuda.synchronize()
     assert torch.equal(dev.cpu(), host)
     s.close()
+
+
+@pytest.mark.parametrize("nx", [80, 192])
+def test_large_column_blocks_at_odd_addresses(L, nx):
+    """Either side of the size where a block at an odd address goes to the
+    copy engine (80 columns of 192 x 96 x 80 in FP16: 66 MB, of twice the depth
+    132 MB; whole lattices 159 and 319 MB): the same bytes at any address, out
+    and back."""
+    import torch
+    for Lz in (80, 160):
+        p = L.Params(Lx=192, Ly=96, Lz=Lz, R=16.0, Uw=0.02, eta_M=0.5, precision=1)
+        rho = 0.5 + np.random.default_rng(Lz).uniform(-0.1, 0.1, (2, Lz, 96, 192))
+        s = L.Solver(p)
+        s.init(0, rho)
+        n = s.columns_bytes(0, nx)
+        want = torch.empty(n, dtype=torch.uint8, device="cuda")
+        s.get_columns(0, 0, nx, want.data_ptr())
+        buf = torch.zeros(n + 16, dtype=torch.uint8, device="cuda")
+        s.get_columns(0, 0, nx, buf.data_ptr() + 1)
+        torch.cuda.synchronize()
+        assert torch.equal(buf[1:1 + n], want) and not buf[:1].any() and not buf[1 + n:].any()
+        s.step(1)
+        s.set_columns(0, 0, nx, buf.data_ptr() + 1)
+        back = torch.empty_like(want)
+        s.get_columns(0, 0, nx, back.data_ptr())
+        torch.cuda.synchronize()
+        assert torch.equal(back, want)
+        s.close()
