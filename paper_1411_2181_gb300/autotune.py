@@ -4,10 +4,10 @@ The step kernel runs one block per column tile and z-chunk, in one of two
 variants: one cell per thread with tiles of 32 x TY cells (TY = 8, 12 or 16)
 or two x-adjacent cells per thread with 32 x 16 tiles (even Lx only); or in
 three passes over the lattice in memory order.  The variant, tile height and
-chunk depth change speed only (the fields agree to FP32 rounding).  ``tune`` times each candidate on a scratch solver built
-from the same parameters, keeps the fastest, and caches the choice in a JSON
-file keyed by the GPU name, the precision and the lattice sizes of the
-batch.
+chunk depth change speed only (the fields agree to FP32 rounding).  ``tune``
+times each candidate on a scratch solver built from the same parameters, keeps
+the fastest, and caches the choice in a JSON file keyed by the GPU name, the
+precision and the lattice sizes of the batch.
 """
 from __future__ import annotations
 
@@ -77,7 +77,13 @@ def tune(params: Params | list[Params], steps: int = 12, cache: str | None = CAC
             s.init(k, r)
         trials = []
         for kern, ty, zc in candidates(plist) + [PASSES]:
-            s.tune(ty, zc, kern)
+            try:
+                s.tune(ty, zc, kern)
+            except lbfe.LbfeError as e:
+                # a handle that cannot run the passes keeps to the tiles
+                if (kern, ty, zc) != PASSES or e.status != lbfe.ERR_BAD_PARAM:
+                    raise
+                continue
             s.step(2)
             e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
             e0.record(stream)

@@ -201,3 +201,60 @@ def test_cases_at_a_larger_gap():
     assert abs(p64.eta_M - p40.eta_M) < 1e-12 and abs(p64.eta_P - p40.eta_P) < 1e-12
     # the emulsion time (in steps) grows with W at a fixed wall speed
     assert abs(study.tau_em(c64) / study.tau_em(c40) - 64 / 40) < 1e-12
+
+
+@pytest.mark.parametrize("refuse", [False, True])
+def test_autotune_without_the_three_pass_kernel(monkeypatch, tmp_path, refuse):
+    """A handle that refuses the three-pass kernel is tuned over the tile
+    shapes alone; any other refusal still shows."""
+    import contextlib
+    import torch
+    from paper_1411_2181_gb300 import autotune, lbfe
+    from paper_1411_2181_gb300.params import Params
+
+    class Event:
+        def __init__(self, enable_timing=False):
+            pass
+
+        def record(self, stream):
+            self.shape = Solver.shape
+
+        def synchronize(self):
+            pass
+
+        def elapsed_time(self, other):
+            return 1.0 + 0.1 * other.shape[1] + 0.01 * other.shape[2] - (2.0 if other.shape[0] == 2 else 0.0)
+
+    class Solver:
+        shape, refused = None, (lbfe.STEP_PASSES, lbfe.ERR_BAD_PARAM)
+
+        def __init__(self, plist, device=None, stream=None):
+            pass
+
+        def init(self, k, r):
+            pass
+
+        def tune(self, ty, zc, kern):
+            if refuse and kern == Solver.refused[0]:
+                raise lbfe.LbfeError(Solver.refused[1], "lbfe_tune")
+            Solver.shape = (kern, ty, zc)
+
+        def step(self, n):
+            pass
+
+        def close(self):
+            pass
+
+    monkeypatch.setattr(lbfe, "Solver", Solver)
+    monkeypatch.setattr(torch.cuda, "get_device_name", lambda dev: "gpu")
+    monkeypatch.setattr(torch.cuda, "Stream", lambda dev=None: None)
+    monkeypatch.setattr(torch.cuda, "stream", lambda s: contextlib.nullcontext())
+    monkeypatch.setattr(torch.cuda, "Event", Event)
+    p = Params(Lx=64, Ly=32, Lz=24, R=4.0)
+    best = autotune.tune(p, cache=str(tmp_path / "a.json"))
+    assert (best["kernel"], best["tile_y"], best["z_chunk"]) == ((0, 8, 0) if refuse else (2, 8, 0))
+    assert len(best["trials"]) == len(autotune.candidates([p])) + (0 if refuse else 1)
+    if refuse:
+        for Solver.refused in ((lbfe.STEP_PASSES, lbfe.ERR_NO_MEMORY), (lbfe.STEP_PAIR, lbfe.ERR_BAD_PARAM)):
+            with pytest.raises(lbfe.LbfeError):
+                autotune.tune(p, cache=None)
