@@ -226,9 +226,6 @@ cudaError_t launch_encode_pop(const LaunchCtx &c, int k, int cur, int s, int i, 
 cudaError_t launch_columns(const LaunchCtx &c, int k, int cur, int x0, int nx, void *block, bool get);
 cudaError_t launch_observables(const InstDev &I, int precision, int cur, unsigned *status, cudaStream_t stream);
 
-// Whether [p, p + bytes) lies in one allocation of device dev (lbfe_capi.cu).
-bool device_range(const void *p, size_t bytes, int dev);
-
 // Host-side droplet analysis (lbfe_analysis.cu): from the observables
 // kernel's per-plane sums prof[6][Lx], fill L_p, L_p/2R, necks, fragments,
 // broken, volume, centroid, M, D and theta of out.

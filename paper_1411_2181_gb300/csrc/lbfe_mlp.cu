@@ -24,6 +24,11 @@
 #include "../../include/lbfe_mlp.h"
 #include "lbfe_internal.cuh"
 
+namespace lbfe {
+// Whether [p, p + bytes) lies in one allocation of device dev (lbfe_capi.cu).
+bool device_range(const void *p, size_t bytes, int dev);
+}  // namespace lbfe
+
 namespace {
 
 constexpr int kLayers = 5;
