@@ -373,6 +373,14 @@ def roofline_record(prec: int, ncell: int, ms_per_step: float, workload_name: st
             "traffic_source": os.path.relpath(prof_file, ROOT) if (prof_file and traffic_per_lup) else None}
 
 
+def launch_record(s, steps: int):
+    """Launch shape of solver ``s`` with the kernel that ``steps`` steps in one
+    call run on, and the number of kernel launches of that call (the
+    three-pass kernel takes up to 16 steps in a launch)."""
+    launch = dict(s.launch_config(), kernel=s.step_variant(steps))
+    return launch, s.launches_per_step() * (-(-steps // 16) if launch["kernel"] == 2 else steps)
+
+
 def time_form(name: str, prec: int, steps: int, warmup: int, device: str, autotune_on: bool):
     """One sub-record: the workload `name` in storage form `prec`, autotuned,
     timed on its own stream with CUDA events (state resident in HBM)."""
@@ -390,7 +398,7 @@ def time_form(name: str, prec: int, steps: int, warmup: int, device: str, autotu
             s.init(k, r)
         ms = timed_steps(s, stream, steps, warmup)
         st = s.check()
-        launch = s.launch_config()
+        launch, _ = launch_record(s, steps)
         s.close()
     del s
     torch.cuda.empty_cache()
@@ -445,9 +453,7 @@ def run_ours(a):
         with ClockSampler(local) as clk:
             ms = timed_steps(s, stream, a.steps, a.warmup, dist)
         st = s.check()
-        launch = s.launch_config()
-        # the three-pass kernel takes up to 16 steps in a launch
-        launches = s.launches_per_step() * (-(-a.steps // 16) if launch["kernel"] == 2 else a.steps)
+        launch, launches = launch_record(s, a.steps)
         status = lbfe._lib.lbfe_status_str(st).decode()
         s.close()
     t_max = reduce_max_ms(ms, device=f"cuda:{local}")

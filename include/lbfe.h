@@ -252,11 +252,16 @@ typedef enum {
  * LBFE_ERR_BAD_PARAM for an unsupported combination.  Synchronises the
  * stream. */
 lbfe_status lbfe_tune(lbfe_handle *h, int step_kernel, int tile_y, int z_chunk);
-/* Current launch shape of the tile kernels (any output may be NULL): kernel
- * variant, tile height, z-chunk of instance 0, persistent grid size and number
- * of work items. */
+/* Launch shape that lbfe_tune set, or a new handle's (any output may be NULL):
+ * kernel variant, tile height, z-chunk of instance 0, persistent grid size and
+ * number of work items.  The last four are the tile kernels', which a handle
+ * keeps beside LBFE_STEP_PASSES.  A new handle's variant is LBFE_STEP_CELL also
+ * where it takes the passes by itself: lbfe_step_variant tells what runs. */
 lbfe_status lbfe_launch_config(const lbfe_handle *h, int *step_kernel, int *tile_y, int *z_chunk, int *grid,
                                int *items);
+/* The variant (lbfe_step_kernel) that lbfe_step(h, nsteps) launches now; -1 for
+ * h = NULL or nsteps < 0. */
+int lbfe_step_variant(const lbfe_handle *h, long long nsteps);
 
 /* Test hook for the failure path of the step kernel (no counterpart in the
  * paper).  what = LBFE_INJECT_SHORT_COPIES: the TMA tensor maps of the

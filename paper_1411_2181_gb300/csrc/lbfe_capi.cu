@@ -371,6 +371,12 @@ bool device_range(const void *p, size_t bytes, int dev) {
 }
 }  // namespace lbfe
 
+// Whether nsteps steps in one call run in three passes, not in tiles.
+static bool takes_passes(const lbfe_handle *h, long long nsteps) {
+    (void)nsteps;
+    return h->passes && !(h->inject & LBFE_INJECT_SHORT_COPIES);
+}
+
 extern "C" {
 
 const char *lbfe_status_str(lbfe_status s) {
@@ -567,7 +573,7 @@ lbfe_status lbfe_step(lbfe_handle *h, long long nsteps) {
     CK(cudaStreamIsCapturing(h->stream, &cs));
     const bool graphs = nsteps >= 2 && cs == cudaStreamCaptureStatusNone;
     const lbfe::LaunchCtx c = h->ctx();
-    if (h->passes && !(h->inject & LBFE_INJECT_SHORT_COPIES)) {
+    if (takes_passes(h, nsteps)) {
         for (long long t = 0; t < nsteps;) {
             const int m = (int)std::min<long long>(lbfe::passes_steps(), nsteps - t);
             CK(lbfe::launch_passes(c, h->cur, m));
@@ -811,6 +817,11 @@ lbfe_status lbfe_launch_config(const lbfe_handle *h, int *step_kernel, int *tile
     if (grid) *grid = h->fused_grid;
     if (items) *items = h->total_items;
     return LBFE_OK;
+}
+
+int lbfe_step_variant(const lbfe_handle *h, long long nsteps) {
+    if (!h || nsteps < 0) return -1;
+    return takes_passes(h, nsteps) ? LBFE_STEP_PASSES : h->step_kernel;
 }
 
 unsigned lbfe_crc32(const void *data, size_t n, unsigned crc) {

@@ -76,6 +76,8 @@ _lib.lbfe_tune.argtypes = [_H, ct.c_int, ct.c_int, ct.c_int]
 _lib.lbfe_tune.restype = ct.c_int
 _lib.lbfe_launch_config.argtypes = [_H] + [ct.POINTER(ct.c_int)] * 5
 _lib.lbfe_launch_config.restype = ct.c_int
+_lib.lbfe_step_variant.argtypes = [_H, ct.c_longlong]
+_lib.lbfe_step_variant.restype = ct.c_int
 _lib.lbfe_test_inject.argtypes = [_H, ct.c_uint]
 _lib.lbfe_test_inject.restype = ct.c_int
 _lib.lbfe_save.argtypes = [_H, ct.c_int, ct.c_char_p]
@@ -214,7 +216,13 @@ class Solver:
         STEP_PASSES (tile_y 8, z_chunk 0)."""
         _check(_lib.lbfe_tune(self._h, int(kernel), int(tile_y), int(z_chunk)), "lbfe_tune")
 
+    def step_variant(self, n: int = 1) -> int:
+        """The kernel (STEP_CELL, STEP_PAIR or STEP_PASSES) that step(n) runs on."""
+        return _lib.lbfe_step_variant(self._h, int(n))
+
     def launch_config(self) -> dict:
+        """Launch shape that tune set, or a new solver's (lbfe_launch_config);
+        step_variant tells which kernel runs."""
         v = [ct.c_int() for _ in range(5)]
         _check(_lib.lbfe_launch_config(self._h, *[ct.byref(x) for x in v]), "lbfe_launch_config")
         return dict(kernel=v[0].value, tile_y=v[1].value, z_chunk=v[2].value, grid=v[3].value, items=v[4].value)

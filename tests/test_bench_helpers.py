@@ -4,6 +4,8 @@ profiled DRAM traffic, and the autotuner summary in the JSON line."""
 import os
 import shutil
 
+import pytest
+
 import bench
 
 
@@ -56,3 +58,21 @@ def test_autotune_summary_keeps_the_fastest_chunk_per_shape():
     s = bench.autotune_summary(shape)["best_ms_per_step"]
     assert s == {"cell_32x8": 0.142, "cell_32x12": 0.141, "pair_32x16": 0.2}
     assert bench.autotune_summary(None) is None
+
+
+@pytest.mark.parametrize("variant,steps,launches", [(0, 20, 40), (1, 3, 6), (2, 1, 2), (2, 16, 2), (2, 17, 4), (2, 200, 26)])
+def test_launches_of_the_kernel_that_runs(variant, steps, launches):
+    """The line names the kernel that ran, also where the handle chose it by
+    itself, and counts its launches (two groups of instances here)."""
+    class Solver:
+        def launch_config(self):
+            return {"kernel": 0, "tile_y": 8}
+
+        def step_variant(self, n):
+            assert n == steps
+            return variant
+
+        def launches_per_step(self):
+            return 2
+
+    assert bench.launch_record(Solver(), steps) == ({"kernel": variant, "tile_y": 8}, launches)

@@ -250,3 +250,41 @@ def test_a_handle_steps_again_after_expired_waits(L, prec):
         same(L, s, ref, len(shapes))
     s.close()
     ref.close()
+
+
+def test_which_kernel_runs(L):
+    """A handle tells which kernel its steps run on: the estimate's choice for
+    new handles (small, ragged and FP16 boxes; the tile kernel on 192 x 96 x 80
+    and 128 x 96 x 80), what lbfe_tune said for tuned ones, the tiles under the
+    short-copies hook.  The default tile shape stays what it is."""
+    for shape, prec, kern in [((32, 32, 32), 0, L.STEP_PASSES), ((32, 32, 32), 1, L.STEP_PASSES),
+                              ((141, 75, 53), 0, L.STEP_PASSES), ((141, 75, 53), 2, L.STEP_PASSES),
+                              ((100, 96, 80), 1, L.STEP_PASSES), ((192, 96, 80), 0, L.STEP_CELL),
+                              ((192, 96, 80), 1, L.STEP_CELL), ((192, 96, 80), 2, L.STEP_CELL),
+                              ((128, 96, 80), 0, L.STEP_CELL)]:
+        s = L.Solver(params(L, shape, prec, 0, 1))
+        assert s.step_variant(20) == kern, (shape, prec)
+        assert s.launch_config()["kernel"] == L.STEP_CELL
+        s.tune(8, 0, L.STEP_PASSES)
+        assert s.step_variant(20) == s.step_variant(1) == s.launch_config()["kernel"] == L.STEP_PASSES
+        s.test_inject(L.INJECT_SHORT_COPIES)
+        assert s.step_variant(20) == L.STEP_CELL
+        s.test_inject(0)
+        s.tune(16, 0, L.STEP_CELL)
+        assert s.step_variant(20) == s.step_variant(1) == L.STEP_CELL
+        s.close()
+    assert L._lib.lbfe_step_variant(None, 1) == -1
+
+
+@pytest.mark.parametrize("prec", [0, 1, 2])
+def test_default_tiles_are_the_passes(L, prec):
+    """The shape a new handle steps a large lattice with (8 rows, 12 with
+    2-byte storage, rows copied by TMA) against the passes, bit for bit."""
+    shape = (192, 96, 80)
+    p = params(L, shape, prec, 0, 1)
+    st = [random_populations(shape, seed=2, amp=0.01)]
+    a, b = solver(L, p, None, st), solver(L, p, (8, 0, L.STEP_PASSES), st)
+    assert a.step_variant(5) == L.STEP_CELL
+    a.step(5)
+    b.step(5)
+    same(L, a, b)
