@@ -381,6 +381,12 @@ def launch_record(s, steps: int):
     return launch, s.launches_per_step() * (-(-steps // 16) if launch["kernel"] == 2 else steps)
 
 
+def observables_bytes(ps) -> int:
+    """Bytes that the observables of every instance bring to the host: six sums
+    a plane, two masses and the status word, 64 bits each."""
+    return sum((6 * p.Lx + 3) * 8 for p in ps)
+
+
 def time_form(name: str, prec: int, steps: int, warmup: int, device: str, autotune_on: bool):
     """One sub-record: the workload `name` in storage form `prec`, autotuned,
     timed on its own stream with CUDA events (state resident in HBM)."""
@@ -482,7 +488,7 @@ def run_ours(a):
             t1 = time.perf_counter()
             s2.close()
         e2e_mlups = ncell * a.steps / (t1 - t0) / 1e6 * world
-        obs_bytes = sum(6 * p.Lx * 8 + 2 * 8 + 4 for p in ps)
+        obs_bytes = observables_bytes(ps)
         e2e = {"value": round(e2e_mlups, 2), "unit": METRIC,
                "h2d_bytes_per_step": int(sum(h.numel() for h in hosts) * 8 / a.steps),
                "d2h_bytes_per_step": int(obs_bytes / a.steps),

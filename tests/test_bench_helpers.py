@@ -76,3 +76,14 @@ def test_launches_of_the_kernel_that_runs(variant, steps, launches):
             return 2
 
     assert bench.launch_record(Solver(), steps) == ({"kernel": variant, "tile_y": 8}, launches)
+
+
+def test_observables_bytes():
+    """As many as lbfe_observables copies: the record of obs_words(Lx) words
+    without its last, the kernel's own counter."""
+    import re
+    from types import SimpleNamespace
+    src = open(os.path.join(bench.ROOT, "paper_1411_2181_gb300", "csrc", "lbfe_internal.cuh")).read()
+    per, const = map(int, re.search(r"obs_words\(int Lx\) \{ return (\d+) \* \(size_t\)Lx \+ (\d+); \}", src).groups())
+    ps = [SimpleNamespace(Lx=192), SimpleNamespace(Lx=33)]
+    assert bench.observables_bytes(ps) == 8 * sum(per * p.Lx + const - 1 for p in ps)
