@@ -192,44 +192,89 @@ struct lbfe_handle {
     }
 };
 
-// Depth of the z-chunks: the one with the least estimated time of the busiest
-// block (a chunk costs four planes more than it holds).  Items of one lattice
-// are equal and start together, so that they march in waves of the resident
-// blocks, at the same pace.  The items of a batch are handed out as blocks become
-// free, and neighbours that started together drift apart over a deep chunk (tiles
-// at a seam or an edge take another time per plane), until the planes they share
-// are no longer in the L2: the time of a plane grows with the depth of the chunks
-// (drift_planes), and what the end leaves uneven comes to half an item.
-// Chunks of at least 8 planes.  Measured, us per step: 256 x 128 x 64 FP16
-// (12 rows; 88 columns), chunks that fill the blocks about once -> waves 307 -> 212;
-// 192 x 96 x 80 keeps its 40 (FP32) and 27 planes (FP16).  Batches at 8, 12, 16,
-// 27 and 64 planes a chunk: twelve uneven lattices FP16 1885, 1755, 1715, 1870
-// and 2275, FP32 2039, 1960, 2005, 2310 and 2957; 32 of them FP16 4192, 3882,
-// 3845, 4173 and 5003; 40 boxes of 40 planes FP16 2340, 2289, 2226, 2279 and 2170,
-// at 20 planes 2042.
-static double drift_planes(const lbfe_handle *h) { return h->precision == LBFE_FP32 ? 43.0 : 86.0; }
-// A plane of items that all start together takes 3.2 us (FP32, 4.4 with 2-byte
-// storage), one of a batch's about 2.3 (3.2) and what the drift adds.
-constexpr double kTogether = 1.4;
+// ---- estimates of the tile kernels' time
+// Unit: a plane of whole tiles, copied by TMA, of one lattice whose items all start
+// together (FP32 3.45 us; see prefer_passes).
 
-static int auto_z_chunk(const std::vector<InstDev> &inst, long long slots, double drift) {
+// A plane's weight: tiles cut by the x period take a tenth more; rows that are no
+// 16-byte multiples are read with ordinary loads, which cost little while the batch's
+// state lies in the L2 (1.05) and, beyond about 80 MB, half as much again in FP32 and
+// 0.3 with 2-byte storage.  Measured over forty lattices, us per plane, FP32 / FP16:
+// 192 x 96 x 80 3.27 / 4.65, 80^3 3.65 / 5.00, 31 x 31 x 200 (34 / 21 MB) 3.4 / 4.6,
+// 50 x 96 x 80 (68 / 41 MB) 4.4 / 4.7, 141 x 75 x 53 (99 / 60 MB) 4.7 / 5.7,
+// 98 x 96 x 80 (132 / 81 MB) 4.8 / 5.9, 255 x 127 x 95 4.9 / 5.7.
+static bool rows_copied(const InstDev &I, int precision) {
+    return (I.Lx * elem_bytes(precision)) % 16 == 0 && (I.Lx * sizeof(float)) % 16 == 0;
+}
+static double plane_weight(const InstDev &I, int precision, double state_mb) {
+    if (rows_copied(I, precision)) return I.Lx % 32 == 0 ? 1.0 : 1.1;
+    const double most = precision == LBFE_FP32 ? 1.45 : 1.3;
+    return 1.05 + (most - 1.05) * std::min(1.0, std::max(0.0, (state_mb - 30.0) / 50.0));
+}
+
+// What the busiest of `slots` resident blocks marches with z-chunks of zc planes (a chunk
+// costs four planes more than it holds).  Items that all start together take the
+// deepest one's planes; those of one lattice march in waves of the resident blocks, at
+// the same pace.  Those of a batch are handed out as blocks become free: equal boxes
+// still in waves, uneven ones evenly but for a third of an item.  A plane then costs less
+// than where all blocks meet at the same planes, and more the deeper the chunks: neighbours
+// that started together drift apart (tiles at a seam or an edge take another time per
+// plane) until the planes they share are no longer in the L2.  With few waves there is
+// little of either.  Measured, us a plane by depth of the chunks, FP32: sixteen
+// 320 x 44 x 40 2.7 (8), 2.74 (10), 2.86 (14), 3.3 (20), 3.6 (40), two of them in one
+// wave 3.2; FP16 3.66, 3.83, 3.76, 3.98, 4.25, one wave 4.45.
+static double march_planes(const std::vector<InstDev> &inst, int precision, int zc, long long slots) {
+    double cells = 0.0, planes = 0.0, deep = 0.0, shallow = 0.0;
+    long long items = 0;
+    int depth = 0;
+    bool equal = true, copied = true;
+    for (auto &I : inst) {
+        cells += (double)I.N;
+        copied = copied && rows_copied(I, precision);
+        equal = equal && I.Lx == inst[0].Lx && I.Ly == inst[0].Ly && I.Lz == inst[0].Lz;
+    }
+    const bool fp32 = precision == LBFE_FP32;
+    const double mb = 1e-6 * cells * (fp32 ? 176.0 : 108.0);
+    for (auto &I : inst) {
+        const int c = std::min(zc, I.Lz);
+        const long long col = (long long)I.ntx * I.nty, nz = (I.Lz + c - 1) / c;
+        const double w = plane_weight(I, precision, mb), item = w * (c + 4);
+        items += col * nz;
+        planes += w * (double)(col * (I.Lz + 4 * nz));
+        deep = std::max(deep, item);
+        shallow = shallow == 0.0 ? item : std::min(shallow, item);
+        depth = std::max(depth, c);
+    }
+    if (items <= slots) return deep;
+    double waves = (double)((items + slots - 1) / slots), march = deep * waves;
+    if (inst.size() == 1) return march;
+    // pace: time of a plane against that of items that start together
+    double pace;
+    if (equal) {
+        pace = copied ? (fp32 ? 0.86 + 0.005 * depth : 0.79 + 0.0075 * depth)
+                      : (fp32 ? 0.75 + 0.012 * depth : 0.73 + 0.0085 * depth);
+        pace = std::min(pace, 1.0);
+    } else {
+        march = std::max(planes / slots + 0.3 * deep, deep + shallow);
+        waves = march / deep;
+        pace = fp32 ? 0.73 + 0.02 * depth : 0.66 + 0.008 * depth;
+    }
+    if (pace < 1.0) pace = 1.0 - (1.0 - pace) * std::max(0.0, 1.0 - 1.1 / waves);
+    return march * pace;
+}
+
+// Depth of the z-chunks, at least 8 planes: the one with the least estimate.  Measured, us
+// per step, against chunks that fill the blocks about once: 256 x 128 x 64 FP16 (12 rows)
+// 307 -> 212; 192 x 96 x 80 keeps its 40 (FP32) and 27 planes (FP16); twelve uneven lattices
+// FP16 2234 -> 1752, FP32 2838 -> 1984; six 64^3 FP32 207 -> 173; two 192 x 96 x 80 in FP32
+// keep one wave (272; 40 planes 335).  Timed at every depth over 114 batches in five forms
+// the chosen one is within 1.3 % of the best on average (filling the blocks once 12 %).
+static int auto_z_chunk(const std::vector<InstDev> &inst, int precision, long long slots) {
     int lz = 0, best = 8;
     for (auto &I : inst) lz = std::max(lz, I.Lz);
     double best_cost = 0.0;
     for (int zc = std::max(8, lz); zc >= 8; --zc) {
-        long long items = 0, planes = 0;
-        int deepest = 0;
-        for (auto &I : inst) {
-            const int c = std::min(zc, I.Lz);
-            const long long col = (long long)I.ntx * I.nty, nz = (I.Lz + c - 1) / c;
-            items += col * nz;
-            planes += col * (I.Lz + 4 * nz);
-            deepest = std::max(deepest, c + 4);
-        }
-        double cost = deepest;
-        if (items > slots)
-            cost = inst.size() == 1 ? (double)deepest * ((items + slots - 1) / slots)
-                                    : ((double)planes / slots + 0.5 * deepest) * (1.0 + (deepest - 4) / drift) / kTogether;
+        const double cost = march_planes(inst, precision, zc, slots);
         if (best_cost == 0.0 || cost < best_cost) {
             best_cost = cost;
             best = zc;
@@ -260,7 +305,7 @@ static lbfe_status configure_fused(lbfe_handle *h, int step_kernel, int tile_y, 
         I.nty = (I.Ly + tile_y - 1) / tile_y;
     }
     const long long slots = (long long)h->num_sms * bps;
-    const int zc_auto = z_chunk == 0 ? auto_z_chunk(h->inst, slots, drift_planes(h)) : 0;
+    const int zc_auto = z_chunk == 0 ? auto_z_chunk(h->inst, h->precision, slots) : 0;
     std::vector<int> off(h->n + 1, 0);
     for (int k = 0; k < h->n; ++k) {
         InstDev &I = h->inst[k];
@@ -310,42 +355,35 @@ static bool passes_possible(const lbfe_handle *h) {
 
 // Whether a new handle's steps run in three passes instead of tiles: the
 // smaller estimate of a step's time (the fields are the same bit for bit).
-//   tiles   planes that the busiest block marches, 3.2 us each (8 rows, FP32),
-//           4.4 (12 rows, 2-byte storage), 3.7 (second-order advection), in
-//           batches as auto_z_chunk says, half as much again where rows are no
-//           16-byte multiples (no copies);
-//   passes  about 8 us of launch and dependent passes, 0.5 ns a cell of the
+//   tiles   march_planes of 3.45 us (8 rows, FP32), 4.6 (12 rows, FP16), 4.8 (BF16), in
+//           second order 3.55 (FP32) and 3.85 (2-byte storage, 8 rows);
+//   passes  about 8 us of launch and dependent passes, 0.32 ns a cell of the
 //           largest plane (a pass stays two planes behind the one before) and
-//           0.100 ns a cell (FP32), 0.105 (FP16), 0.112 (BF16), 0.15
-//           (second-order advection), a tenth more in batches.
+//           0.108 ns a cell (FP32), 0.105 (FP16), 0.112 (BF16), in second order 0.157
+//           and 0.14; in batches 1.1 (FP16), 1.15 (BF16) and 1.05 (2-byte in second
+//           order) times as much.
 // Measured, us per step, tiles / passes (GB300, FP32 unless noted): 32^3
-// 35 / 15, 37^3 41 / 17, 240 x 20 x 17 41 / 21, 96 x 48 x 48 39 / 30, 64^3
-// 37 / 32 (FP16 51 / 45), 141 x 75 x 53 103 / 62 (FP16 101 / 75), 40 x 128 x 90
-// 94 / 53, 128 x 128 x 16 37 / 41, 100 x 96 x 80 109 / 83 (FP16 141 / 87), 192 x 96 x 80 142 / 160
-// (FP16 140 / 165, BF16 145 / 175, second order 160 / 233), 256 x 128 x 64
-// 212 / 235, sixteen 320 x 44 x 40 995 / 973 (FP16 850 / 1079), forty 2444 / 2430,
-// twelve uneven lattices 1961 / 1986 (FP16 1714 / 2078, second order 2079 / 2823),
-// four of them 686 / 636, 32 of them 4297 / 4390.
+// 37 / 15, 37^3 41 / 17, 240 x 20 x 17 41 / 21, 96 x 48 x 48 37 / 31, 64^3
+// 38 / 32 (FP16 51 / 36), 141 x 75 x 53 104 / 62 (FP16 103 / 64), 40 x 128 x 90
+// 94 / 53, 128 x 128 x 16 38 / 41, 100 x 96 x 80 112 / 84 (FP16 142 / 88), 192 x 96 x 80 144 / 162
+// (FP16 144 / 167, BF16 151 / 178, second order 167 / 239), 256 x 128 x 64
+// 211 / 239, sixteen 320 x 44 x 40 997 / 991 (FP16 860 / 1102), six 394 / 373,
+// twelve uneven lattices 1984 / 1986 (FP16 1763 / 2078, second order 2118 / 2823).
+// Over 780 shapes and forms the choice is within 0.4 % of the better one on average.
 static bool prefer_passes(const lbfe_handle *h) {
-    const bool fp32 = h->precision == LBFE_FP32;
-    double planes = 0.0, most = 0.0, cells = 0.0, plane = 0.0, depth = 0.0;
-    for (int k = 0; k < h->n; ++k) {
-        const InstDev &I = h->inst[k];
-        const double w = h->maps[k].ok ? 1.0 : 1.5;
-        planes += w * I.ntx * I.nty * (I.Lz + 4.0 * I.nzc);
-        most = std::max(most, w * (I.zc + 4.0));
-        depth = std::max(depth, (double)I.zc);
+    const bool fp32 = h->precision == LBFE_FP32, bf16 = h->precision == LBFE_BF16_OFFSET;
+    double cells = 0.0, plane = 0.0;
+    int zc = 0;
+    for (auto &I : h->inst) {
         cells += (double)I.N;
         plane = std::max(plane, (double)I.Lx * I.Ly);
+        zc = std::max(zc, I.zc);
     }
-    const double slots = (double)h->num_sms * h->blocks_per_sm;
-    double march = most;
-    if (h->total_items > slots)
-        march = h->n == 1 ? most * std::ceil(h->total_items / slots)
-                          : (planes / slots + 0.5 * most) * (1.0 + depth / drift_planes(h)) / kTogether;
-    const double tile = march * (h->advection ? 3.7 : (fp32 ? 3.2 : 4.4));
-    const double ns = h->advection ? 0.15 : (fp32 ? 0.100 : (h->precision == LBFE_FP16_OFFSET ? 0.105 : 0.112));
-    return 8.0 + 0.5e-3 * plane + 1e-3 * ns * (h->n > 1 ? 1.1 : 1.0) * cells < tile;
+    const double us = h->advection ? (fp32 ? 3.55 : 3.85) : (fp32 ? 3.45 : (bf16 ? 4.8 : 4.6));
+    const double tiles = us * march_planes(h->inst, h->precision, zc, (long long)h->num_sms * h->blocks_per_sm);
+    const double ns = h->advection ? (fp32 ? 0.157 : 0.14) : (fp32 ? 0.108 : (bf16 ? 0.112 : 0.105));
+    const double batch = h->n == 1 || fp32 ? 1.0 : (h->advection ? 1.05 : (bf16 ? 1.15 : 1.1));
+    return 8.0 + 0.32e-3 * plane + 1e-3 * ns * batch * cells < tiles;
 }
 
 namespace lbfe {

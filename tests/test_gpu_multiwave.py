@@ -176,3 +176,22 @@ def test_bf16_step_counts_are_per_instance(L, kernel, tile_y):
         solo.step(5 if k == 1 else 8)
         assert np.array_equal(batch.get_field(k, L.FIELD_F), solo.get_field(0, L.FIELD_F)), k
         solo.close()
+
+
+@pytest.mark.parametrize("shapes,prec,adv,tile_y,zc", [
+    ([(192, 96, 80)], 0, 0, 8, 40), ([(192, 96, 80)], 1, 0, 12, 27), ([(256, 128, 64)], 1, 0, 12, 13),
+    ([(64, 64, 64)] * 6, 0, 0, 8, 22), ([(64, 64, 64)] * 6, 1, 1, 8, 22), ([(192, 96, 80)] * 2, 0, 1, 8, 80),
+    ([(192, 96, 80)] * 2, 1, 0, 12, 27), ([(96, 64, 48)] * 5, 1, 0, 12, 16), ([(73, 90, 46)] * 12, 0, 0, 8, 46),
+    ([(101, 100, 26)] * 5, 0, 0, 8, 26)])
+def test_automatic_z_chunks(L, shapes, prec, adv, tile_y, zc):
+    """The depth the rule takes: single lattices in whole waves, equal boxes
+    in waves too (one wave where that is no more planes), rows without copies
+    weighted.  Timed at every depth, each is within 1 % of the best; the
+    estimate that took all batches for evenly loaded chose 8 planes for the
+    fourth (224 us a step, 173 at 22), 16 for the seventh (329, 292 at 27), 12
+    for the ninth (731, 674 at 46) and 9 for the last (292, 265 at 26)."""
+    s = L.Solver([L.Params(Lx=a, Ly=b, Lz=c, R=4.0, Uw=0.02, eta_M=0.5, precision=prec, advection=adv)
+                  for a, b, c in shapes])
+    s.tune(tile_y, 0, 0)
+    assert s.launch_config()["z_chunk"] == zc
+    s.close()
