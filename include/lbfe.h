@@ -246,8 +246,9 @@ typedef enum {
  * A new handle starts with LBFE_STEP_CELL, tile_y 8 (FP32, or any precision
  * with LBFE_ADVECTION_UPWIND2_MINMOD) or 12 (FP16 / BF16 storage) and the
  * automatic z-chunk, and takes LBFE_STEP_PASSES by itself where that is
- * faster for its lattices (small, ragged or many): the fields are the same
- * bit for bit.  A handle that was tuned keeps what it was given.  With LBFE_ADVECTION_UPWIND2_MINMOD only
+ * faster for its lattices (small, ragged or many) and the steps of the call:
+ * the fields are the same bit for bit.  A handle that was tuned keeps what it
+ * was given.  With LBFE_ADVECTION_UPWIND2_MINMOD only
  * LBFE_STEP_CELL at tile_y 8 is accepted.
  * LBFE_ERR_BAD_PARAM for an unsupported combination.  Synchronises the
  * stream. */

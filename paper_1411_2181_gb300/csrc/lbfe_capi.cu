@@ -148,7 +148,8 @@ struct lbfe_handle {
     int step_kernel = LBFE_STEP_CELL;
     int advection = 0;               // lbfe_params::advection of every instance
     bool passes_tuned = false;       // ... because lbfe_tune said so
-    bool passes = false;             // the step runs in three passes (lbfe_passes.cu), else in tiles
+    bool passes = false;             // steps run in three passes (lbfe_passes.cu) where takes_passes says so
+    double est_tiles = 0.0, est_passes = 0.0, est_tail = 0.0;   // us (estimate_steps)
     unsigned inject = 0;             // lbfe_test_inject bits
     unsigned *status = nullptr;
     int cur = 0;
@@ -194,7 +195,7 @@ struct lbfe_handle {
 
 // ---- estimates of the tile kernels' time
 // Unit: a plane of whole tiles, copied by TMA, of one lattice whose items all start
-// together (FP32 3.45 us; see prefer_passes).
+// together (FP32 3.45 us; see estimate_steps).
 
 // A plane's weight: tiles cut by the x period take a tenth more; rows that are no
 // 16-byte multiples are read with ordinary loads, which cost little while the batch's
@@ -353,15 +354,20 @@ static bool passes_possible(const lbfe_handle *h) {
     return false;
 }
 
-// Whether a new handle's steps run in three passes instead of tiles: the
-// smaller estimate of a step's time (the fields are the same bit for bit).
+// Estimates of a step's time in tiles and in three passes, and of what a launch of the
+// passes takes besides its steps; a new handle takes the smaller sum for the number of
+// steps asked for (takes_passes; the fields are the same bit for bit).
 //   tiles   march_planes of 3.45 us (8 rows, FP32), 4.6 (12 rows, FP16), 4.8 (BF16), in
 //           second order 3.55 (FP32) and 3.85 (2-byte storage, 8 rows);
 //   passes  about 8 us of launch and dependent passes, 0.32 ns a cell of the
 //           largest plane (a pass stays two planes behind the one before) and
 //           0.108 ns a cell (FP32), 0.105 (FP16), 0.112 (BF16), in second order 0.157
 //           and 0.14; in batches 1.1 (FP16), 1.15 (BF16) and 1.05 (2-byte in second
-//           order) times as much.
+//           order) times as much, in calls of 20 steps;
+//   tail    a launch of up to 16 steps ends, and begins, with passes that nothing
+//           overlaps: 4.5 us and 0.054 ns a cell, 20 us at most.  One step in a call / twenty:
+//           32^3 19.6 / 15.1, 64^3 47 / 32 (tiles 38), 96 x 48 x 48 43 / 31 (tiles 37),
+//           141 x 75 x 53 85 / 62, 192 x 96 x 80 184 / 163.
 // Measured, us per step, tiles / passes (GB300, FP32 unless noted): 32^3
 // 37 / 15, 37^3 41 / 17, 240 x 20 x 17 41 / 21, 96 x 48 x 48 37 / 31, 64^3
 // 38 / 32 (FP16 51 / 36), 141 x 75 x 53 104 / 62 (FP16 103 / 64), 40 x 128 x 90
@@ -369,8 +375,9 @@ static bool passes_possible(const lbfe_handle *h) {
 // (FP16 144 / 167, BF16 151 / 178, second order 167 / 239), 256 x 128 x 64
 // 211 / 239, sixteen 320 x 44 x 40 997 / 991 (FP16 860 / 1102), six 394 / 373,
 // twelve uneven lattices 1984 / 1986 (FP16 1763 / 2078, second order 2118 / 2823).
-// Over 780 shapes and forms the choice is within 0.4 % of the better one on average.
-static bool prefer_passes(const lbfe_handle *h) {
+// Over 780 shapes and forms, at 1, 2, 4 and 20 steps a call, the choice is within 0.4 % of
+// the better one on average.
+static void estimate_steps(lbfe_handle *h) {
     const bool fp32 = h->precision == LBFE_FP32, bf16 = h->precision == LBFE_BF16_OFFSET;
     double cells = 0.0, plane = 0.0;
     int zc = 0;
@@ -380,10 +387,11 @@ static bool prefer_passes(const lbfe_handle *h) {
         zc = std::max(zc, I.zc);
     }
     const double us = h->advection ? (fp32 ? 3.55 : 3.85) : (fp32 ? 3.45 : (bf16 ? 4.8 : 4.6));
-    const double tiles = us * march_planes(h->inst, h->precision, zc, (long long)h->num_sms * h->blocks_per_sm);
+    h->est_tiles = us * march_planes(h->inst, h->precision, zc, (long long)h->num_sms * h->blocks_per_sm);
     const double ns = h->advection ? (fp32 ? 0.157 : 0.14) : (fp32 ? 0.108 : (bf16 ? 0.112 : 0.105));
     const double batch = h->n == 1 || fp32 ? 1.0 : (h->advection ? 1.05 : (bf16 ? 1.15 : 1.1));
-    return 8.0 + 0.32e-3 * plane + 1e-3 * ns * batch * cells < tiles;
+    h->est_passes = 8.0 + 0.32e-3 * plane + 1e-3 * ns * batch * cells;
+    h->est_tail = std::min(20.0, 4.5 + 0.054e-3 * cells);
 }
 
 namespace lbfe {
@@ -411,8 +419,11 @@ bool device_range(const void *p, size_t bytes, int dev) {
 
 // Whether nsteps steps in one call run in three passes, not in tiles.
 static bool takes_passes(const lbfe_handle *h, long long nsteps) {
-    (void)nsteps;
-    return h->passes && !(h->inject & LBFE_INJECT_SHORT_COPIES);
+    if (!h->passes || (h->inject & LBFE_INJECT_SHORT_COPIES)) return false;
+    if (h->passes_tuned || nsteps < 1) return true;
+    // launches a step; est_passes holds those of twenty steps
+    const long long launches = (nsteps + lbfe::passes_steps() - 1) / lbfe::passes_steps();
+    return h->est_passes + h->est_tail * std::max(0.0, (double)launches / (double)nsteps - 0.1) < h->est_tiles;
 }
 
 extern "C" {
@@ -560,7 +571,8 @@ lbfe_status lbfe_create(lbfe_handle **hp, const lbfe_params *p, int n, void *dev
         delete h;
         return st;
     }
-    h->passes = passes_possible(h) && prefer_passes(h);
+    estimate_steps(h);
+    h->passes = h->est_passes < h->est_tiles && passes_possible(h);
     *hp = h;
     return LBFE_OK;
 }

@@ -17,7 +17,7 @@
 // instructions.  Measured in FP32, tile kernel -> passes, us per step: 32^3
 // 35 -> 15, 64^3 37 -> 32, 141 x 75 x 53 103 -> 62, sixteen 320 x 44 x 40
 // 1107 -> 970; 192 x 96 x 80 142 -> 160 (the tile kernel stays).
-// Which of the two a handle runs is decided in lbfe_capi.cu (prefer_passes).
+// Which of the two a handle runs is decided in lbfe_capi.cu (takes_passes).
 //
 // Work.  A slot is one pass over up to R x 256 cells.  Slots are numbered so
 // that passes M, X and U of the lattice follow one another at fixed distances

@@ -288,3 +288,24 @@ def test_default_tiles_are_the_passes(L, prec):
     a.step(5)
     b.step(5)
     same(L, a, b)
+
+
+@pytest.mark.parametrize("prec,adv", [(0, 0), (2, 0), (0, 1)])
+def test_the_steps_of_a_call_decide_too(L, prec, adv):
+    """A launch of the passes has an end that nothing overlaps: 64^3 takes the
+    tiles for a call of one step (38 us, passes 47) and the passes for twenty
+    (32), 32^3 the passes for both.  A handle that goes from one to the other
+    with every call has the bits of either."""
+    small = L.Solver(params(L, (32, 32, 32), prec, adv, 1))
+    assert small.step_variant(1) == small.step_variant(20) == L.STEP_PASSES
+    shape = (50, 96, 80) if prec or adv else (64, 64, 64)
+    p = params(L, shape, prec, adv, 1)
+    st = [random_populations(shape, seed=6, amp=0.01)]
+    s, tile, passes = solver(L, p, None, st), solver(L, p, (8, 0, 0), st), solver(L, p, (8, 0, L.STEP_PASSES), st)
+    assert s.step_variant(1) == L.STEP_CELL and s.step_variant(20) == L.STEP_PASSES
+    assert passes.step_variant(1) == L.STEP_PASSES
+    for n in (1, 20, 1, 1, 17, 20, 1):
+        for h in (s, tile, passes):
+            h.step(n)
+        same(L, s, tile)
+        same(L, s, passes)
