@@ -116,3 +116,21 @@ def test_reduced_storage_with_second_order_advection(L, prec):
         s.close()
     scale = np.abs(out[0]).max()
     assert np.abs(out[1] - out[0]).max() <= (2e-3 if prec == 1 else 2e-2) * scale
+
+
+def test_tile_kernel_500_steps(L):
+    """The 500 steps on the tile kernel, whichever kernel a new handle takes
+    for 32^3: the same bits."""
+    p, rho, steps = configs.config1()
+    p = replace(p, advection=1)
+    out = []
+    for tune in (None, (8, 0, L.STEP_CELL)):
+        s = L.Solver(p)
+        if tune:
+            s.tune(*tune)
+            assert s.step_variant(steps) == L.STEP_CELL
+        s.init(0, rho)
+        s.step(steps)
+        out.append([s.get_field(0, w) for w in (L.FIELD_F, L.FIELD_C)])
+        s.close()
+    assert all(np.array_equal(a, b) for a, b in zip(*out))

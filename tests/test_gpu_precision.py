@@ -135,3 +135,22 @@ def test_full_lattice_reduced_storage_10k_steps(L):
         print(f"full lattice, precision {prec} vs FP32, {steps} steps: max |dD| {dD:.2e}, "
               f"max |dtheta| {dth:.3f} deg, mass {dm:.2e}")
         assert dD < tol_D and dth < tol_theta and dm < tol_mass, (prec, dD, dth, dm)
+
+
+@pytest.mark.parametrize("prec", [0, 1, 2])
+def test_tile_kernel_over_the_same_run(L, runs, prec):
+    """The 3000 steps on the tile kernel (the shape of a new handle's tiles),
+    whichever kernel a new handle takes for this lattice: the same masses,
+    sums and angles, digit for digit, and so the same distance from the
+    oracle."""
+    p, rho, _ = configs.config3(crop=True)
+    s = L.Solver(replace(p, precision=prec))
+    s.tune(8 if prec == 0 else 12, 0, L.STEP_CELL)
+    assert s.step_variant(EVERY) == L.STEP_CELL
+    s.init(0, rho)
+    out = [s.observables(0)]
+    for _ in range(STEPS // EVERY):
+        s.step(EVERY)
+        out.append(s.observables(0))
+    assert out == runs[prec]
+    s.close()
