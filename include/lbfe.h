@@ -242,14 +242,15 @@ typedef enum {
 
 /* Launch shape of the step kernel: variant (lbfe_step_kernel), column-tile
  * height tile_y (tile width 32; 16 for LBFE_STEP_PAIR) and z-chunk depth in
- * planes (0 = automatic: fill the resident blocks of the GPU about once).
+ * planes (0 = automatic: the depth with the least estimated time for the
+ * lattices of the handle, at least 8).
  * A new handle starts with LBFE_STEP_CELL, tile_y 8 (FP32, or any precision
  * with LBFE_ADVECTION_UPWIND2_MINMOD) or 12 (FP16 / BF16 storage) and the
  * automatic z-chunk, and takes LBFE_STEP_PASSES by itself where that is
  * faster for its lattices (small, ragged or many) and the steps of the call:
  * the fields are the same bit for bit.  A handle that was tuned keeps what it
- * was given.  With LBFE_ADVECTION_UPWIND2_MINMOD only
- * LBFE_STEP_CELL at tile_y 8 is accepted.
+ * was given.  With LBFE_ADVECTION_UPWIND2_MINMOD only LBFE_STEP_CELL at
+ * tile_y 8 and LBFE_STEP_PASSES are accepted.
  * LBFE_ERR_BAD_PARAM for an unsupported combination.  Synchronises the
  * stream. */
 lbfe_status lbfe_tune(lbfe_handle *h, int step_kernel, int tile_y, int z_chunk);

@@ -15,8 +15,9 @@
 // lattice of few columns still fills the GPU.  They pay with the populations'
 // second read (the L2 serves part of it), 40 bytes a cell of scratch and more
 // instructions.  Measured in FP32, tile kernel -> passes, us per step: 32^3
-// 35 -> 15, 64^3 37 -> 32, 141 x 75 x 53 103 -> 62, sixteen 320 x 44 x 40
-// 1107 -> 970; 192 x 96 x 80 142 -> 160 (the tile kernel stays).
+// 37 -> 15, 64^3 38 -> 32, 141 x 75 x 53 104 -> 62, sixteen 320 x 44 x 40
+// 997 -> 991; 192 x 96 x 80 144 -> 162 (the tile kernel stays), in calls of
+// twenty steps.
 // Which of the two a handle runs is decided in lbfe_capi.cu (takes_passes).
 //
 // Work.  A slot is one pass over up to R x 256 cells.  Slots are numbered so

@@ -212,7 +212,8 @@ class Solver:
 
     def tune(self, tile_y: int = 8, z_chunk: int = 0, kernel: int = 0):
         """Launch shape of the step: kernel STEP_CELL (tile_y in 8, 12, 16) or
-        STEP_PAIR (tile_y 16, even Lx), and the z-chunk depth (0 = auto), or
+        STEP_PAIR (tile_y 16, even Lx), and the z-chunk depth (0 = the depth
+        with the least estimated time), or
         STEP_PASSES (tile_y 8, z_chunk 0)."""
         _check(_lib.lbfe_tune(self._h, int(kernel), int(tile_y), int(z_chunk)), "lbfe_tune")
 
