@@ -25,7 +25,7 @@ CACHE = os.path.join(os.path.dirname(os.path.abspath(__file__)), "_build", "auto
 
 def _key(params: list[Params], gpu: str) -> str:
     dims = ";".join(f"{p.Lx}x{p.Ly}x{p.Lz}" for p in params)
-    return f"{gpu}|v3|prec{params[0].precision}|adv{params[0].advection}|n{len(params)}|{dims}"
+    return f"{gpu}|v4|prec{params[0].precision}|adv{params[0].advection}|n{len(params)}|{dims}"
 
 
 def _load(path):
